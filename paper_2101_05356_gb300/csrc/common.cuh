@@ -88,12 +88,17 @@ struct LightDev {
     int type, env;
 };
 
-// Binary BVH node holding both children's boxes (64 B, four 16-B loads).
+// Binary BVH node (96 B): both children's boxes and child codes (64 B, four
+// 16-B loads), then each child's plane bound (two more, read by the any-hit
+// traversal): every point x of the child's triangles has n . x <= h, n the
+// child's mean normal (k_planes).
 struct __align__(16) BvhNode {
     float4 a;   // lo0.x lo0.y lo0.z hi0.x
     float4 b;   // hi0.y hi0.z lo1.x lo1.y
     float4 c;   // lo1.z hi1.x hi1.y hi1.z
     int4 d;     // child0, child1 (>= 0 internal, < 0 leaf ~slot), pad, pad
+    float4 p0;  // n0.x n0.y n0.z h0
+    float4 p1;  // n1.x n1.y n1.z h1
 };
 
 struct DevScene {
@@ -180,7 +185,7 @@ struct BvhScratch {
     int* parent_int;     // [T - 1]
     int* parent_leaf;    // [T]
     int* flag;           // [T - 1]
-    float4* box_int;     // [2 (T - 1)] lo, hi
+    float4* box_int;     // [2 (T - 1)] lo, hi; w: first leaf slot, leaf count (int bits)
     float4* box_leaf;    // [2 T]
     unsigned* aabb;      // [6] ordered-int scene bounds
 };

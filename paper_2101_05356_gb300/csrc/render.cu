@@ -26,15 +26,16 @@ constexpr int RT_WARPS = RT_THREADS / 32;
 #define FR_STACK_LOCAL 1
 #endif
 // minimum resident blocks per SM requested from the compiler (register cap).
-// Measured on GB300 (paper-scale face): the forward is fastest at 10 blocks
-// (3.11 ms; 8: 3.28 ms, 12: 3.47 ms), the primary-edge kernel at 8, the
+// Measured on GB300 (paper-scale face): the forward is fastest at 9 blocks
+// (1.39 ms; 8: 1.42 ms, 10: 1.40 ms, 12: 1.88 ms), the primary-edge kernel at 6
+// (0.39 ms beside the adjoint; 7: 0.43 ms, 8: 0.46 ms, 9: 0.50 ms), the
 // adjoint reading hit records at 5 (0.601 ms; 6: 0.618 ms, 8: 0.637 ms) and
 // the re-tracing adjoint at 8 (4.20 ms; 6: 4.38 ms, 5: 4.65 ms).
 #ifndef FR_FWD_MIN_BLOCKS
-#define FR_FWD_MIN_BLOCKS 10
+#define FR_FWD_MIN_BLOCKS 9
 #endif
 #ifndef FR_EDGE_MIN_BLOCKS
-#define FR_EDGE_MIN_BLOCKS 8
+#define FR_EDGE_MIN_BLOCKS 6
 #endif
 #ifndef FR_ADJ_REC_MIN_BLOCKS
 #define FR_ADJ_REC_MIN_BLOCKS 5
