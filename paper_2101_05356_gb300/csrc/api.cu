@@ -243,6 +243,8 @@ DevItem make_item(const fr_ctx* c, int k, const ItemArgs& a) {
         it.B.vals = c->topo_vals;
         it.B.keys = nullptr;
     }
+    s.parent_leaf = it.B.parent_leaf;
+    s.parent_int = it.B.parent_int;
     it.nodes = sl.nodes;
     it.tris = sl.tris;
     it.slot_of = sl.slot_of;

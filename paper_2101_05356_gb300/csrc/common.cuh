@@ -111,6 +111,8 @@ struct DevScene {
     const BvhNode* nodes;   // [max(T - 1, 1)]
     const float4* tris;     // [3T] triangles in BVH leaf order; tris[3s].w = id bits
     const int* slot_of;     // [T] leaf slot of each triangle (inverse of the leaf order)
+    const int* parent_leaf; // [T] parent node of each leaf slot (-1: the tree is one leaf)
+    const int* parent_int;  // [T - 1] parent of each internal node (not read for the root)
     const LightDev* lights; // [NL]
     const float* stage;     // [NL][12] virtual light stage frame (centre, unit face V0 V1 V2);
                             // non-null when the lights are built from (d, a, p) parameters

@@ -26,13 +26,13 @@ constexpr int RT_WARPS = RT_THREADS / 32;
 #define FR_STACK_LOCAL 1
 #endif
 // minimum resident blocks per SM requested from the compiler (register cap).
-// Measured on GB300 (paper-scale face): the forward is fastest at 9 blocks
-// (1.39 ms; 8: 1.42 ms, 10: 1.40 ms, 12: 1.88 ms), the primary-edge kernel at 6
+// Measured on GB300 (paper-scale face): the forward is fastest at 8 blocks
+// (1.25 ms; 7: 1.30 ms, 9: 1.27 ms, 6: 1.37 ms), the primary-edge kernel at 6
 // (0.39 ms beside the adjoint; 7: 0.43 ms, 8: 0.46 ms, 9: 0.50 ms), the
 // adjoint reading hit records at 5 (0.601 ms; 6: 0.618 ms, 8: 0.637 ms) and
 // the re-tracing adjoint at 8 (4.20 ms; 6: 4.38 ms, 5: 4.65 ms).
 #ifndef FR_FWD_MIN_BLOCKS
-#define FR_FWD_MIN_BLOCKS 9
+#define FR_FWD_MIN_BLOCKS 8
 #endif
 #ifndef FR_EDGE_MIN_BLOCKS
 #define FR_EDGE_MIN_BLOCKS 6
@@ -163,11 +163,12 @@ FR_D bool light_visible_geometry(const LightDev& L, float3 z, const SampleState&
     return dot(ss.ns, lv) > 0.0f && -dot(L.n, lv) > 0.0f;
 }
 
-// Trace the queued jobs [head, head + n) of this warp's ring (lane k takes job k).
+// Trace the queued jobs [head, head + n) of this warp's ring (lane k takes job
+// k) from the warp's cover, or from the root (NoCover).
 // ENV: the launch may hold environment blocks (lights at infinity); otherwise
 // their code is compiled out.
-template <bool ENV>
-FR_D void drain(const DevScene& S, WarpQueue& q, int head, int n, Stack st, RayStats& rs) {
+template <bool ENV, class C>
+FR_D void drain(const DevScene& S, WarpQueue& q, const C& cover, int head, int n, Stack st, RayStats& rs) {
     const int lane = threadIdx.x & 31;
     if (lane < n) {
         const float4 a = q.job[(head + lane) & 63][0], b = q.job[(head + lane) & 63][1];
@@ -177,7 +178,7 @@ FR_D void drain(const DevScene& S, WarpQueue& q, int head, int n, Stack st, RayS
         // to a light at infinity
         const bool distant = ENV && ((tag >> 16) & 1);
         const RayPre r = ray_setup(y, distant ? z : z - y);
-        if (!trace_any(S, r, SHADOW_EPS, distant ? INFINITY : 1.0f - SHADOW_EPS, skip, st, rs))
+        if (!trace_any(S, cover, r, SHADOW_EPS, distant ? INFINITY : 1.0f - SHADOW_EPS, skip, st, rs))
             atomicOr(&q.vis[tag & 31], 1ull << ((tag >> 8) & 63));
     }
     __syncwarp();
@@ -186,9 +187,9 @@ FR_D void drain(const DevScene& S, WarpQueue& q, int head, int n, Stack st, RayS
 // Warp-cooperative shadow visibility for the lights [j0, j0 + 64): bit j - j0
 // is set when the shadow ray to this lane's light-j sample is traced and
 // unoccluded.  All 32 lanes must call this together.
-template <bool ENV>
+template <bool ENV, class C>
 FR_D uint64_t shadow_mask(const DevScene& S, const SampleState& ss, const Sampler& smp, int dim0,
-                          WarpQueue& q, Stack st, RayStats& rs, int j0) {
+                          WarpQueue& q, const C& cover, Stack st, RayStats& rs, int j0) {
     const int lane = threadIdx.x & 31;
     q.vis[lane] = 0ull;
     __syncwarp();
@@ -196,11 +197,13 @@ FR_D uint64_t shadow_mask(const DevScene& S, const SampleState& ss, const Sample
     int head = 0, count = 0;
     DimCache dc;
     const int j1 = min(S.NL, j0 + 64);
-    for (int j = j0; j < j1; ++j) {
+    // light by light, then (j = j1) what is left in the ring: one place that
+    // traces, so the kernel holds its code once
+    for (int j = j0; j <= j1; ++j) {
         bool need = false;
         float3 z = f3(0.0f, 0.0f, 0.0f);
-        const bool distant = ENV && S.lights[j].type == FR_LIGHT_ENV_D;      // warp-uniform
-        if (want) {
+        const bool distant = ENV && j < j1 && S.lights[j].type == FR_LIGHT_ENV_D;      // warp-uniform
+        if (want && j < j1) {
             const LightDev& L = S.lights[j];
             const float2 u = dc.pair(smp, dim0 + 2 * j);
             if (distant) {                       // z = the direction of the sample
@@ -220,13 +223,13 @@ FR_D uint64_t shadow_mask(const DevScene& S, const SampleState& ss, const Sample
         }
         count += __popc(ballot);
         __syncwarp();
-        if (count >= 32) {
-            drain<ENV>(S, q, head, 32, st, rs);
-            head = (head + 32) & 63;
-            count -= 32;
+        if (count >= 32 || (j == j1 && count > 0)) {
+            const int n = min(count, 32);
+            drain<ENV>(S, q, cover, head, n, st, rs);
+            head = (head + n) & 63;
+            count -= n;
         }
     }
-    if (count > 0) drain<ENV>(S, q, head, count, st, rs);
     return q.vis[lane];
 }
 
@@ -345,14 +348,20 @@ FR_D float3 radiance_from(const DevScene& S, const DevParams& P, const SampleSta
 
 // Warp-cooperative visibility at screen point (sx, sy): the camera ray's hit
 // (without the material) and both shadow-visibility words.
-template <bool ENV>
+FR_D void make_cover(const DevScene&, const SampleState&, NoCover&) {}
+FR_D void make_cover(const DevScene& S, const SampleState& ss, Cover& c) {
+    build_cover(S, c, __ballot_sync(FULL, ss.hit && ss.lit), ss.slot);
+}
+
+template <bool ENV, class C>
 FR_D void visibility_at(const DevScene& S, const DevParams& P, bool active, float sx, float sy,
-                        const Sampler& smp, int dim0, RtShared& sh, Stack stk, SampleState& ss, uint64_t* vis,
-                        RayStats& rs) {
+                        const Sampler& smp, int dim0, RtShared& sh, C& cover, Stack stk, SampleState& ss,
+                        uint64_t* vis, RayStats& rs) {
     primary_state<true, false>(S, P, active, sx, sy, stk, ss, rs);
+    make_cover(S, ss, cover);
     vis[0] = vis[1] = 0ull;
     for (int j0 = 0; j0 < max(S.NL, 1); j0 += 64)            // lights in chunks of 64 (warp-uniform)
-        vis[j0 >> 6] = shadow_mask<ENV>(S, ss, smp, dim0, sh.wq[threadIdx.x >> 5], stk, rs, j0);
+        vis[j0 >> 6] = shadow_mask<ENV>(S, ss, smp, dim0, sh.wq[threadIdx.x >> 5], cover, stk, rs, j0);
 }
 
 // Radiance of a sample whose visibility is known: the material, then the lights.
@@ -372,7 +381,8 @@ template <bool ENV>
 FR_D float3 radiance_at(const DevScene& S, const DevParams& P, bool active, float sx, float sy,
                         const Sampler& smp, int dim0, RtShared& sh, Stack stk, SampleState& ss, uint64_t* vis,
                         RayStats& rs) {
-    visibility_at<ENV>(S, P, active, sx, sy, smp, dim0, sh, stk, ss, vis, rs);
+    NoCover root;
+    visibility_at<ENV>(S, P, active, sx, sy, smp, dim0, sh, root, stk, ss, vis, rs);
     return shade_visible<ENV>(S, P, smp, dim0, ss, vis);
 }
 
@@ -426,8 +436,9 @@ __global__ void __launch_bounds__(RT_THREADS, FR_FWD_MIN_BLOCKS) k_forward(const
     SampleState ss;
     uint64_t vis[2];
     RayStats rs;
+    __shared__ Cover cover[RT_WARPS];
     visibility_at<ENV>(S, P, valid, (float)(pixel % S.W) + jit.x, (float)(pixel / S.W) + jit.y, smp, 2, sh,
-                       my_stack(sh), ss, vis, rs);
+                       cover[threadIdx.x >> 5], my_stack(sh), ss, vis, rs);
     if (records_only) {                                 // launch-uniform
         flush_stats(S.counters + 3, rs);                // the adjoint's rays
         if (valid) {
@@ -565,8 +576,8 @@ FR_D void shadow_edge_env(const DevScene& S, const DevParams& P, const LightDev&
     float3 wp = wv + m * SHADOW_EPS, wm = wv - m * SHADOW_EPS;
     wp = wp * (1.0f / length(wp));
     wm = wm * (1.0f / length(wm));
-    const bool vp = !trace_any(S, ray_setup(ss.y, wp), SHADOW_EPS, INFINITY, ss.slot, st, rs);
-    const bool vm = !trace_any(S, ray_setup(ss.y, wm), SHADOW_EPS, INFINITY, ss.slot, st, rs);
+    const bool vp = !trace_any(S, NoCover{}, ray_setup(ss.y, wp), SHADOW_EPS, INFINITY, ss.slot, st, rs);
+    const bool vm = !trace_any(S, NoCover{}, ray_setup(ss.y, wm), SHADOW_EPS, INFINITY, ss.slot, st, rs);
     const float dV = (float)vp - (float)vm;
     if (dV == 0.0f) return;
     const float3 Le = env_radiance(P, row * L.env + col);
@@ -622,8 +633,8 @@ FR_D void shadow_edge(const DevScene& S, const DevParams& P, const EdgeLists& EL
     if (!(tl > 0.0f)) return;
     const float3 m = cross(L.n, tan) * (1.0f / tl);
     const float3 zp = z + m * SHADOW_EPS, zm = z - m * SHADOW_EPS;
-    const bool vp = !trace_any(S, ray_setup(ss.y, zp - ss.y), SHADOW_EPS, 1.0f - SHADOW_EPS, ss.slot, st, rs);
-    const bool vm = !trace_any(S, ray_setup(ss.y, zm - ss.y), SHADOW_EPS, 1.0f - SHADOW_EPS, ss.slot, st, rs);
+    const bool vp = !trace_any(S, NoCover{}, ray_setup(ss.y, zp - ss.y), SHADOW_EPS, 1.0f - SHADOW_EPS, ss.slot, st, rs);
+    const bool vm = !trace_any(S, NoCover{}, ray_setup(ss.y, zm - ss.y), SHADOW_EPS, 1.0f - SHADOW_EPS, ss.slot, st, rs);
     const float dV = (float)vp - (float)vm;
     if (dV == 0.0f) return;
     const float3 I = intensity(S, P, j);
@@ -755,7 +766,7 @@ __global__ void __launch_bounds__(RT_THREADS, RECORDED ? FR_ADJ_REC_MIN_BLOCKS :
             if (recorded)
                 vis_w[j0 >> 6] = (valid && ss.hit) ? it.rec_vis[vis_words(S) * ql + (j0 >> 6)] : 0ull;
             else
-                vis_w[j0 >> 6] = shadow_mask<ENV>(S, ss, smp, 2, sh.wq[threadIdx.x >> 5], my_stack(sh), rs, j0);
+                vis_w[j0 >> 6] = shadow_mask<ENV>(S, ss, smp, 2, sh.wq[threadIdx.x >> 5], NoCover{}, my_stack(sh), rs, j0);
         }
     }
     sample_material(S, P, ss);
@@ -1454,7 +1465,7 @@ FR_D void spec_eval(const DevItem& it, const SpecQueue& q, int head, int n, int 
     if (ss.hit) ss.lit = front;
     uint64_t vis[2] = {0ull, 0ull};
     for (int j0 = 0; j0 < max(S.NL, 1); j0 += 64)                  // warp-uniform
-        vis[j0 >> 6] = shadow_mask<ENV>(S, ss, smp, 4, sh.wq[threadIdx.x >> 5], stk, rs, j0);
+        vis[j0 >> 6] = shadow_mask<ENV>(S, ss, smp, 4, sh.wq[threadIdx.x >> 5], NoCover{}, stk, rs, j0);
     float3 Lp = f3(0.0f, 0.0f, 0.0f), Lm = f3(0.0f, 0.0f, 0.0f);
     if (active && ss.hit) {
         sample_material(S, P, ss);

@@ -69,3 +69,38 @@ def test_visibility_equals_brute_force(n, scale, flat):
         agree = (vis | ~same) if flat else (vis & same)
         assert np.sum(~agree) <= 2, int(np.sum(~agree))
         assert r.status() == 0
+
+
+def _with_far_chain(n, steps):
+    """The soup with single triangles outside the view at distances 8^k along +-x, +-y and behind the camera: each
+    split of the tree takes off few of them, so the soup's leaves lie deep."""
+    sc, pr = _soup(n, 1.0, False)
+    far = []
+    for k in range(steps):
+        d = 6.0 * 8.0 ** k
+        for ax, sg in ((0, 1), (0, -1), (1, 1), (1, -1), (2, 1)):
+            c = np.zeros(3)
+            c[ax] = sg * d
+            c[2] += 1.0
+            far.append(c + 0.05 * d * np.array([[0, 0, 0], [1, 0, 0.3], [0, 1, 0.6]]))
+    v = np.concatenate([sc.mean, np.concatenate(far)])
+    m = len(v)
+    return scenes.make(v, np.arange(m).reshape(-1, 3), np.zeros((1, m, 3)), sc.lights, width=24, height=24, spp=4)[0], pr
+
+
+@pytest.mark.parametrize("n,steps", [(40, 3), (3000, 12), (3000, 14)])
+def test_cover_of_deep_leaves(n, steps):
+    """A warp's shadow rays start from the siblings of a leaf's ancestors, at most 23 of them; deeper leaves keep the
+    topmost ones and the path's node below them."""
+    from paper_2101_05356_gb300 import facert
+    sc, pr = _with_far_chain(n, steps)
+    _, ot, om = oracle.render(sc, pr, records=True)
+    r = facert.Renderer(sc)
+    dp = r.device_params(pr)
+    out = torch.zeros(3, dtype=torch.int32, device="cuda")
+    facert.fr_debug_bvh(r.ctx, dp, out)
+    assert (out.cpu().tolist()[2] > 24) == (n > 1000)
+    _, tri, mask = r.records(dp)
+    agree = (tri.cpu().numpy() == ot) & (mask.cpu().numpy().view(np.uint64) == om).all(axis=1)
+    assert np.sum(~agree) <= 2, int(np.sum(~agree))
+    assert r.status() == 0
