@@ -263,25 +263,33 @@ FR_D void set_status(int* status, int bit) { atomicOr(status, bit); }
 
 // Warp-aggregated fixed-point add of N values that share one key (the
 // channels of one texel, the coordinates of one vertex): one match over the
-// warp, then each value summed over the lanes sharing the key in lane order,
-// and the sums added to addr[n] by the first of those lanes.
+// warp, then a tree over the lanes sharing a key (in each round every second
+// remaining lane takes the next one's values, all groups in step), and the
+// sums added to addr[n] by the group's first lane.  At most five rounds; a loop
+// over a group's lanes, one shuffle each, took as many as its lanes for every
+// group in turn (512 x 512 step, 16 samples a pixel: with warp_sum4 the adjoint
+// 1.36 -> 1.22 ms).
 template <int N>
 FR_D void warp_agg_add_n(fix64* const (&addr)[N], const float (&val)[N], uint32_t key, uint32_t active) {
-    const uint32_t peers = __match_any_sync(active, key);
+    const uint32_t group = __match_any_sync(active, key);
     const int lane = threadIdx.x & 31;
+    uint32_t above = group & (0xfffffffeu << lane);      // the group's lanes after this one
+    uint32_t rank = __popc(group & ((1u << lane) - 1u));
     float sum[N];
 #pragma unroll
-    for (int n = 0; n < N; ++n) sum[n] = 0.0f;
-    uint32_t m = peers;
-    while (m) {
-        const int src = __ffs(m) - 1;
+    for (int n = 0; n < N; ++n) sum[n] = val[n];
+    while (__any_sync(active, above != 0u)) {
+        const int next = above ? __ffs(above) - 1 : lane;
 #pragma unroll
-        for (int n = 0; n < N; ++n) sum[n] += __shfl_sync(peers, val[n], src);
-        m &= m - 1;
+        for (int n = 0; n < N; ++n) {
+            const float v = __shfl_sync(active, sum[n], next);
+            if (above) sum[n] += v;
+        }
+        above &= __ballot_sync(active, !(rank & 1u));    // odd ranks have been taken
+        rank >>= 1;
     }
-    if (lane == __ffs(peers) - 1) {
+    if (lane == __ffs(group) - 1) {
 #pragma unroll
         for (int n = 0; n < N; ++n) fix_add(addr[n], sum[n]);
     }
 }
-

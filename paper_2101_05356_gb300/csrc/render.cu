@@ -392,6 +392,20 @@ FR_D float warp_sum(float v) {
     return v;
 }
 
+// Sums of four values over the warp: value q in lanes [8 q, 8 q + 8).  Two
+// halving steps move each value's terms to its quarter of the lanes, three
+// more add them there: 6 shuffles instead of 20.
+FR_D float warp_sum4(float a, float b, float c, float d) {
+    const int lane = threadIdx.x & 31;
+    const bool h = lane & 16, l = lane & 8;
+    const float u = (h ? c : a) + __shfl_xor_sync(FULL, h ? a : c, 16);     // a | c
+    const float v = (h ? d : b) + __shfl_xor_sync(FULL, h ? b : d, 16);     // b | d
+    float s = (l ? v : u) + __shfl_xor_sync(FULL, l ? u : v, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+    return s;
+}
+
 // sum over aligned groups of `width` lanes (width a power of two <= 32)
 FR_D float group_sum(float v, int width) {
     for (int o = width >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
@@ -831,20 +845,13 @@ __global__ void __launch_bounds__(RT_THREADS, RECORDED ? FR_ADJ_REC_MIN_BLOCKS :
                                                          gl4[0] != 0.0f || gl4[1] != 0.0f || gl4[2] != 0.0f ||
                                                          gl4[3] != 0.0f);
             if (any) {
-                const float sx_ = warp_sum(gI.x), sy_ = warp_sum(gI.y), sz_ = warp_sum(gI.z);
-                if ((threadIdx.x & 31) == 0) {
-                    float* wa = acc_dyn + (threadIdx.x >> 5) * n_acc;
-                    wa[1 + 3 * j] = sx_;
-                    wa[1 + 3 * j + 1] = sy_;
-                    wa[1 + 3 * j + 2] = sz_;
-                }
+                float* wa = acc_dyn + (threadIdx.x >> 5) * n_acc + 1;
+                const float sI = warp_sum4(gI.x, gI.y, gI.z, 0.0f);
+                const int lane = threadIdx.x & 31, q = lane >> 3;
+                if ((lane & 7) == 0 && q < 3) wa[3 * j + q] = sI;
                 if (stage) {                                   // block-uniform
-                    float sg[4];
-                    for (int q = 0; q < 4; ++q) sg[q] = warp_sum(gl4[q]);
-                    if ((threadIdx.x & 31) == 0) {
-                        float* wa = acc_dyn + (threadIdx.x >> 5) * n_acc + 1 + 3 * S.NL + 4 * j;
-                        for (int q = 0; q < 4; ++q) wa[q] = sg[q];
-                    }
+                    const float sg = warp_sum4(gl4[0], gl4[1], gl4[2], gl4[3]);
+                    if ((lane & 7) == 0) wa[3 * S.NL + 4 * j + q] = sg;
                 }
             }
         }
