@@ -327,7 +327,7 @@ FR_D void build_cover(const DevScene& s, Cover& c, unsigned lit, int slot) {
     const int src = (lit >> 16) ? 15 + __ffs(lit >> 16) : 31 - __clz(lit | 1u);    // a middle one
     slot = __shfl_sync(0xffffffffu, slot, src);
     int depth = 0, mine = -1, below = 0;          // lane l keeps ancestor l (mod 32) and its child on the path
-    if (lit && slot >= 0) {
+    if (lit && slot >= 0 && s.T > 1) {            // a single leaf has no parent
         int me = ~slot, node = __ldg(&s.parent_leaf[slot]);
         while (node >= 0 && depth < 128) {
             if ((depth & 31) == lane) {
