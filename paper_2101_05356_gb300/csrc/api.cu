@@ -81,6 +81,7 @@ struct fr_ctx {
     LinearModel albedo[2];                     // diffuse, specular; rows 3 M^2 (optional)
     bool have_albedo = false;
     // static SAH topology of the mesh (refitted per call unless FR_FLAG_LBVH)
+    RefitTopology refit{};
     int *topo_child = nullptr, *topo_parent_int = nullptr, *topo_parent_leaf = nullptr, *topo_vals = nullptr;
     int* landmarks = nullptr;                  // landmark vertex indices [n_landmarks]
     int n_landmarks = 0;
@@ -241,7 +242,6 @@ DevItem make_item(const fr_ctx* c, int k, const ItemArgs& a) {
         it.B.parent_int = c->topo_parent_int;
         it.B.parent_leaf = c->topo_parent_leaf;
         it.B.vals = c->topo_vals;
-        it.B.keys = nullptr;
     }
     s.parent_leaf = it.B.parent_leaf;
     s.parent_int = it.B.parent_int;
@@ -416,16 +416,20 @@ fr_status upload_model(fr_ctx* c, LinearModel& m, int rows, int K, const float* 
     return FR_OK;
 }
 
-// stage lights -> morph -> pose -> face normals + Morton keys -> vertex normals -> BVH
+// stage lights -> morph -> pose, vertex normals and BVH
 void build_geometry(fr_ctx* c, int n, cudaStream_t st) {
     bool any_stage = false;
     for (int k = 0; k < n; ++k) any_stage |= c->h_items[k].S.stage != nullptr;
     if (any_stage) launch_stage_lights(c->d_items, n, c->NL, st);
     morph(c, n, st);
+    if (!(c->cfg.flags & FR_FLAG_LBVH)) {
+        launch_pose_refit(c->d_items, n, c->faces, c->vf_off, c->vf_idx, c->refit, c->N, st);
+        return;
+    }
     launch_pose(c->d_items, n, c->N, st);
     launch_faces(c->d_items, n, c->faces, c->T, st);
     launch_vertex_normals(c->d_items, n, c->vf_off, c->vf_idx, c->N, st);
-    launch_lbvh(c->d_items, n, c->faces, c->T, c->status, (c->cfg.flags & FR_FLAG_LBVH) != 0, st);
+    launch_lbvh(c->d_items, n, c->faces, c->T, c->status, st);
 }
 
 fr_status forward_pass(fr_ctx* c, int n, cudaStream_t st) {
@@ -583,6 +587,7 @@ fr_status alloc_slot(fr_ctx* c, Slot& sl) {
     TRY(dalloc(c, &sl.B.box_int, 2 * (size_t)std::max(T - 1, 1)));
     TRY(dalloc(c, &sl.B.box_leaf, 2 * (size_t)T));
     TRY(dalloc(c, &sl.B.aabb, 6));
+    TRY(dalloc(c, &sl.B.treelet_box, 3 * (size_t)c->refit.n_treelets));
     TRY(dalloc(c, &sl.nodes, std::max(T - 1, 1)));
     TRY(dalloc(c, &sl.tris, 3 * (size_t)T));
     TRY(dalloc(c, &sl.slot_of, T));
@@ -764,6 +769,21 @@ fr_status fr_set_mesh(fr_ctx* c, const fr_mesh* m) {
         CK(c, cudaMemcpy(c->topo_parent_leaf, topo.parent_leaf.data(), sizeof(int) * topo.parent_leaf.size(),
                          cudaMemcpyHostToDevice));
         CK(c, cudaMemcpy(c->topo_vals, topo.vals.data(), sizeof(int) * topo.vals.size(), cudaMemcpyHostToDevice));
+        std::vector<int2> runs;
+        std::vector<Treelet> treelets;
+        std::vector<TopNode> tops;
+        build_refit_lists(topo, T, runs, treelets, tops);
+        int2* d_runs = nullptr;
+        Treelet* d_treelets = nullptr;
+        TopNode* d_tops = nullptr;
+        TRY(dalloc(c, &d_runs, runs.size()));
+        TRY(dalloc(c, &d_treelets, treelets.size()));
+        TRY(dalloc(c, &d_tops, tops.size()));
+        CK(c, cudaMemcpy(d_runs, runs.data(), sizeof(int2) * runs.size(), cudaMemcpyHostToDevice));
+        CK(c, cudaMemcpy(d_treelets, treelets.data(), sizeof(Treelet) * treelets.size(), cudaMemcpyHostToDevice));
+        if (!tops.empty())
+            CK(c, cudaMemcpy(d_tops, tops.data(), sizeof(TopNode) * tops.size(), cudaMemcpyHostToDevice));
+        c->refit = RefitTopology{d_runs, d_treelets, d_tops, (int)treelets.size(), (int)tops.size()};
     }
     TRY(dalloc(c, &c->faces, T));
     TRY(dalloc(c, &c->uv, N));

@@ -6,19 +6,9 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "refit.cuh"
 
 namespace {
-
-// R = Rz(t2) Ry(t1) Rx(t0), row-major
-FR_D void euler_R(const float* rot, float R[9]) {
-    float sx, cx, sy, cy, sz, cz;
-    sincosf(rot[0], &sx, &cx);
-    sincosf(rot[1], &sy, &cy);
-    sincosf(rot[2], &sz, &cz);
-    R[0] = cz * cy; R[1] = cz * sy * sx - sz * cx; R[2] = cz * sy * cx + sz * sx;
-    R[3] = sz * cy; R[4] = sz * sy * sx + cz * cx; R[5] = sz * sy * cx - cz * sx;
-    R[6] = -sy;     R[7] = cy * sx;                R[8] = cy * cx;
-}
 
 // Items per k_set_items launch: 32 x 632-byte items stay under the 32 KB
 // kernel-parameter limit.
@@ -90,14 +80,10 @@ __global__ void __launch_bounds__(256) k_pose(const DevItem* items, int N) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < N) {
         const float* vm = it.v_model;
-        const float wx = vm[3 * i] - T[0], wy = vm[3 * i + 1] - T[1], wz = vm[3 * i + 2] - T[2];
-        // v' = R^T w
-        const float x = R[0] * wx + R[3] * wy + R[6] * wz;
-        const float y = R[1] * wx + R[4] * wy + R[7] * wz;
-        const float z = R[2] * wx + R[5] * wy + R[8] * wz;
-        it.v_cam[i] = make_float4(x, y, z, 0.0f);
-        atomicMin(&bmin[0], ordered(x)); atomicMin(&bmin[1], ordered(y)); atomicMin(&bmin[2], ordered(z));
-        atomicMax(&bmax[0], ordered(x)); atomicMax(&bmax[1], ordered(y)); atomicMax(&bmax[2], ordered(z));
+        const float3 p = pose_vertex(R, f3(vm[3 * i] - T[0], vm[3 * i + 1] - T[1], vm[3 * i + 2] - T[2]));
+        it.v_cam[i] = make_float4(p.x, p.y, p.z, 0.0f);
+        atomicMin(&bmin[0], ordered(p.x)); atomicMin(&bmin[1], ordered(p.y)); atomicMin(&bmin[2], ordered(p.z));
+        atomicMax(&bmax[0], ordered(p.x)); atomicMax(&bmax[1], ordered(p.y)); atomicMax(&bmax[2], ordered(p.z));
     }
     __syncthreads();
     if (threadIdx.x < 3) {
@@ -122,7 +108,7 @@ __global__ void __launch_bounds__(256) k_faces(const DevItem* items, const int4*
     const int4 t = faces[f];
     const float4* v = it.v_cam;
     const float3 a = xyz(v[t.x]), b = xyz(v[t.y]), c = xyz(v[t.z]);
-    const float3 n = cross(b - a, c - a);
+    const float3 n = face_normal(a, b, c);
     it.n_face[f] = make_float4(n.x, n.y, n.z, 0.0f);
     const unsigned* aabb = it.B.aabb;
     const float3 lo = f3(unordered(aabb[0]), unordered(aabb[1]), unordered(aabb[2]));
@@ -136,10 +122,8 @@ __global__ void __launch_bounds__(256) k_faces(const DevItem* items, const int4*
         const uint32_t q = min((uint32_t)(u * 1024.0f), 1023u);
         code |= spread10(q) << (2 - k);
     }
-    if (it.B.keys) {                         // Morton keys only for the per-call LBVH rebuild
-        it.B.keys[f] = code;
-        it.B.vals[f] = f;
-    }
+    it.B.keys[f] = code;
+    it.B.vals[f] = f;
 }
 
 // Vertex normal = normalised sum of its faces' un-normalised normals, gathered
@@ -150,10 +134,8 @@ __global__ void __launch_bounds__(256) k_vertex_normals(const DevItem* items, co
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     float3 m = f3(0.0f, 0.0f, 0.0f);
-    for (int k = off[i]; k < off[i + 1]; ++k) m += xyz(it.n_face[idx[k]]);
-    const float len = length(m);
-    const float inv = len > 0.0f ? 1.0f / len : 0.0f;
-    it.vn[i] = make_float4(m.x * inv, m.y * inv, m.z * inv, len);
+    for (int k = off[i]; k < off[i + 1]; ++k) m = add_rn(m, xyz(it.n_face[idx[k]]));
+    it.vn[i] = vertex_normal(m);
 }
 
 // dE/dm_i = (I - n n^T) dE/dn_i / |m_i|
@@ -372,6 +354,7 @@ void launch_stage_lights(const DevItem* items, int n, int NL, cudaStream_t st) {
     fr_count_launches(1);
 }
 
+// The pose of the per-call LBVH rebuild (the static topology's is in refit.cu).
 void launch_pose(const DevItem* items, int n, int N, cudaStream_t st) {
     k_aabb_reset<<<n, 32, 0, st>>>(items);
     k_pose<<<dim3(nb(N, 256), n), 256, 0, st>>>(items, N);

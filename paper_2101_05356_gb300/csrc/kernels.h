@@ -98,10 +98,30 @@ struct BvhTopology {
 };
 void build_bvh_topology(const float* v, const int* faces, int T, BvhTopology& out);
 
-// lbvh.cu: rebuild = Morton sort + Karras radix tree per call; otherwise the
-// items' BvhScratch carries a fixed topology and only the boxes are refitted
-void launch_lbvh(const DevItem* items, int n, const int4* faces, int T, int* status, bool rebuild,
-                 cudaStream_t st);
+// refit.cu: pose, vertex normals and the boxes and plane bounds of the static
+// topology.  A treelet is a subtree of up to 256 leaves; `up` is 2 * parent +
+// side, -1 for the root.
+struct Treelet {
+    int code, first, count, up;          // child code, its run of leaf slots
+};
+struct TopNode {                         // a node above the treelets
+    int node, up, first, count;
+    int treelet, n_treelets;             // its run of treelets
+};
+struct RefitTopology {
+    const int2* runs;                    // [T - 1] each node's first leaf slot and leaf count
+    const Treelet* treelets;
+    const TopNode* tops;
+    int n_treelets, n_tops;
+};
+void build_refit_lists(const BvhTopology& topo, int T, std::vector<int2>& runs, std::vector<Treelet>& treelets,
+                       std::vector<TopNode>& tops);
+void launch_pose_refit(const DevItem* items, int n, const int4* faces, const int* vf_off, const int* vf_idx,
+                       const RefitTopology& topo, int N, cudaStream_t st);
+
+// lbvh.cu: Morton sort + Karras radix tree of the call's geometry (after
+// launch_pose, launch_faces), its boxes and plane bounds
+void launch_lbvh(const DevItem* items, int n, const int4* faces, int T, int* status, cudaStream_t st);
 void launch_bvh_check(const DevItem* items, int T, int* out, cudaStream_t st);
 
 // render.cu

@@ -7,6 +7,7 @@
 // triangles; nodes store both children's boxes for two-wide tests.
 #include "common.cuh"
 #include "kernels.h"
+#include "refit.cuh"
 
 namespace {
 
@@ -169,11 +170,6 @@ __global__ void __launch_bounds__(256) k_karras(const DevItem* items, int n, int
     if (right < 0) parent_leaf[~right] = i; else parent_int[right] = i;
 }
 
-__global__ void k_flag_reset(const DevItem* items, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n - 1) items[blockIdx.y].B.flag[i] = 0;
-}
-
 // flags 0; parents and child codes -1 (an unwritten child reads as leaf 0,
 // never as an ancestor)
 __global__ void k_bvh_init(const DevItem* items, int n) {
@@ -222,11 +218,8 @@ __global__ void __launch_bounds__(256) k_boxes(const DevItem* items, const int4*
     it.slot_of[id] = s;
     tris[3 * s + 1] = make_float4(b.x, b.y, b.z, 0.0f);
     tris[3 * s + 2] = make_float4(c.x, c.y, c.z, 0.0f);
-    float3 lo = f3(fminf(a.x, fminf(b.x, c.x)), fminf(a.y, fminf(b.y, c.y)), fminf(a.z, fminf(b.z, c.z)));
-    float3 hi = f3(fmaxf(a.x, fmaxf(b.x, c.x)), fmaxf(a.y, fmaxf(b.y, c.y)), fmaxf(a.z, fmaxf(b.z, c.z)));
-    // pad so that the FP32 slab test never culls a triangle the exact test hits
-    lo = f3(lo.x - 1e-5f - 1e-6f * fabsf(lo.x), lo.y - 1e-5f - 1e-6f * fabsf(lo.y), lo.z - 1e-5f - 1e-6f * fabsf(lo.z));
-    hi = f3(hi.x + 1e-5f + 1e-6f * fabsf(hi.x), hi.y + 1e-5f + 1e-6f * fabsf(hi.y), hi.z + 1e-5f + 1e-6f * fabsf(hi.z));
+    const Box3 own = padded_box(xyz(a), xyz(b), xyz(c));
+    float3 lo = own.lo, hi = own.hi;
     int first = s, count = 1;                           // a node's leaves are consecutive slots
     box_leaf[2 * s] = make_float4(lo.x, lo.y, lo.z, __int_as_float(first));
     box_leaf[2 * s + 1] = make_float4(hi.x, hi.y, hi.z, __int_as_float(count));
@@ -298,36 +291,23 @@ __global__ void __launch_bounds__(256) k_pack(const DevItem* items, int n) {
 // together a larger one (its leaf slots are consecutive, so lanes read
 // neighbouring triangles).  Lane l of warp w owns node w + l * (number of warps):
 // the large nodes of the pre-order numbering's first chain land in different warps.
-constexpr int PLANE_MAX = 4096, PLANE_THREAD = 8;
+constexpr int PLANE_THREAD = 8;
 
 FR_D float3 area_vector(const float4* tris, int s) {
     const float3 a = xyz(tris[3 * s]);
     return cross(xyz(tris[3 * s + 1]) - a, xyz(tris[3 * s + 2]) - a);
 }
 
-FR_D float3 unit_or_zero(float3 m) {
-    const float l = length(m);
-    return l > 0.0f && l < INFINITY ? m * (1.0f / l) : f3(0.0f, 0.0f, 0.0f);
-}
-
-// (max n . x, max |x| component) over triangle s
 FR_D void plane_reach(const float4* tris, int s, float3 n, float& h, float& mag) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float3 p = xyz(tris[3 * s + k]);
-        h = fmaxf(h, dot(n, p));
-        mag = fmaxf(mag, fmaxf(fabsf(p.x), fmaxf(fabsf(p.y), fabsf(p.z))));
-    }
+    for (int k = 0; k < 3; ++k) plane_height(xyz(tris[3 * s + k]), n, h, mag);
 }
 
 // code >= 0: internal node, < 0: leaf ~slot; the child's record in its parent
 FR_D void store_plane(const BvhScratch& B, BvhNode* nodes, int code, float3 n, float h, float mag) {
     const int p = code < 0 ? B.parent_leaf[~code] : B.parent_int[code];
     if (p < 0) return;                                  // an invalid tree (its status is set): no record
-    const bool flat = n.x == 0.0f && n.y == 0.0f && n.z == 0.0f;
-    // the pad covers the rounding of both sides of the test (a few 2^-24 of the
-    // coordinates' magnitude), as the boxes' does
-    const float4 v = make_float4(n.x, n.y, n.z, flat ? 1.0f : h + 1e-5f + 1e-6f * mag);
+    const float4 v = plane_record(n, h, mag);
     (B.child[2 * p] == code ? nodes[p].p0 : nodes[p].p1) = v;
 }
 
@@ -430,19 +410,7 @@ int nb(long n, int t) { return (int)((n + t - 1) / t); }
 
 }  // namespace
 
-void launch_lbvh(const DevItem* items, int n, const int4* faces, int T, int* status, bool rebuild,
-                 cudaStream_t st) {
-    if (!rebuild) {                                  // refit a fixed topology: reset the climb flags only
-        if (T > 1) {
-            k_flag_reset<<<dim3(nb(T - 1, 256), n), 256, 0, st>>>(items, T);
-            fr_count_launches(1);
-        }
-        k_boxes<<<dim3(nb(T, 256), n), 256, 0, st>>>(items, faces, T, status);
-        k_pack<<<dim3(nb(T > 1 ? T - 1 : 1, 256), n), 256, 0, st>>>(items, T);
-        fr_count_launches(2);
-        launch_planes(items, n, T, st);
-        return;
-    }
+void launch_lbvh(const DevItem* items, int n, const int4* faces, int T, int* status, cudaStream_t st) {
     const int n_tiles = nb(T, SORT_TILE);
     for (int pass = 0; pass < 4; ++pass) {
         const int shift = 8 * pass;
