@@ -1,10 +1,17 @@
 // Fused multi-tensor Adam with the regularisers of the two-stage optimisation
 // (Sec. 4, Eq. loss1 and loss3): shape prior, light prior, soft box
 // constraints (expression, intensities, light-stage geometry, textures),
-// texture symmetry, chromaticity consistency and smoothness.  One
-// launch updates every parameter group of a stage; each thread owns one
-// element, adds the regulariser gradient (texture stencils read neighbours) to
-// the render gradient, and applies the Adam step with per-group learning rate.
+// texture symmetry, chromaticity consistency and smoothness.  Two launches
+// update every parameter group of a stage: the first adds the regulariser
+// gradient (texture stencils read neighbours, so x must not change yet) to the
+// render gradient and updates the moments, a thread to a texel or element; the
+// second applies the Adam step with per-group learning rate.
+//
+// Bound by HBM (x, g, m, v and the references read, m, v and x written: 58 MB
+// for 512 x 512 textures, 8.5 us) and, in the first launch, by the quotients of
+// the chromaticity term.  With one thread per element and the energies in FP64
+// that launch took 103 us there, nearly all of it FP64 instructions; measured
+// now 22 us, and 8 us the second (13.7 us with one element a thread).
 #include "../../include/facert.h"
 #include "common.cuh"
 #include "kernels.h"
@@ -15,7 +22,8 @@ constexpr int ADAM_THREADS = 256;
 
 struct GroupTable {
     fr_opt_group g[FR_MAX_OPT_GROUPS];
-    int block_start[FR_MAX_OPT_GROUPS + 1];
+    int block_start[FR_MAX_OPT_GROUPS + 1];      // first block of each group: moments, update
+    int apply_start[FR_MAX_OPT_GROUPS + 1];
     int n_groups;
     float beta1, beta2, eps;
     float bc1[FR_MAX_OPT_GROUPS], bc2[FR_MAX_OPT_GROUPS];   // bias corrections 1 - beta^t per group
@@ -23,7 +31,8 @@ struct GroupTable {
 
 FR_D float sgnf(float x) { return (float)((x > 0.0f) - (x < 0.0f)); }
 
-// Regulariser gradient and energy contribution of element i of group G.
+// Regulariser gradient and energy contribution of element i of group G (the
+// texture groups: texel_grad).
 FR_D float reg_grad(const fr_opt_group& G, int i, float x, double* energy) {
     float g = 0.0f;
     double e = 0.0;
@@ -100,54 +109,6 @@ FR_D float reg_grad(const fr_opt_group& G, int i, float x, double* energy) {
         }
         break;
     }
-    case FR_GROUP_TEX_RGB:
-    case FR_GROUP_TEX_MONO: {
-        const int C = G.kind == FR_GROUP_TEX_RGB ? 3 : 1;
-        const int M = G.width;
-        const int ch = i % C, t = i / C, col = t % M, row = t / M;
-        const float* X = G.x;
-        if (G.w_smooth != 0.0f) {                  // sum_i sum_{j in N4(i)} |X_j - X_i|^2
-            float s = 0.0f;
-            double es = 0.0;
-            const int nb[4][2] = {{row, col - 1}, {row, col + 1}, {row - 1, col}, {row + 1, col}};
-            for (int k = 0; k < 4; ++k) {
-                const int rr = nb[k][0], cc = nb[k][1];
-                if (rr < 0 || rr >= M || cc < 0 || cc >= M) continue;
-                const float d = x - X[(rr * M + cc) * C + ch];
-                s += d;
-                es += (double)d * d;
-            }
-            g += 4.0f * G.w_smooth * s;
-            e += (double)G.w_smooth * es;              // each ordered pair once here; summed over i
-        }
-        if (G.w_sym != 0.0f) {                     // sum |X(x) - X(flip x)|, flip: column -> M - 1 - column
-            const int fc = M - 1 - col;
-            if (fc != col) {
-                const float d = x - X[(row * M + fc) * C + ch];
-                g += 2.0f * G.w_sym * sgnf(d);
-                e += (double)G.w_sym * fabsf(d);
-            }
-        }
-        if (G.w_chroma != 0.0f && C == 3 && G.aux) {   // sum |kappa(X) - kappa(X0)|, kappa(c) = c / (sum c + 1e-6)
-            const float* p = X + t * 3;
-            const float* q = G.aux + t * 3;
-            const float S = p[0] + p[1] + p[2] + 1e-6f, S0 = q[0] + q[1] + q[2] + 1e-6f;
-            float gc = 0.0f;
-            for (int k = 0; k < 3; ++k) {
-                const float kk = p[k] / S;
-                const float sg = sgnf(kk - q[k] / S0);
-                gc += sg * (((k == ch) ? 1.0f : 0.0f) - kk) / S;
-                if (k == ch) e += (double)G.w_chroma * fabsf(kk - q[k] / S0);
-            }
-            g += G.w_chroma * gc;
-        }
-        if (G.w_box != 0.0f) {                     // soft box [0, 1]
-            const float lo = fminf(x, 0.0f), hi = fmaxf(x - 1.0f, 0.0f);
-            g += 2.0f * G.w_box * (lo + hi);
-            e += (double)G.w_box * (lo * lo + hi * hi);
-        }
-        break;
-    }
     default:
         break;
     }
@@ -155,34 +116,210 @@ FR_D float reg_grad(const fr_opt_group& G, int i, float x, double* energy) {
     return g;
 }
 
+// An unevaluated sum hi + lo of two FP32 numbers: the texture energies are
+// summed in these instead of in FP64, whose pipe takes 64 cycles per warp
+// instruction.  Every term enters exactly (a product with its rounding error,
+// by FMA), and a sum keeps about 48 bits: against a 64-bit evaluation the
+// energies are as far off as with FP64 sums (4e-8, the FP32 differences that
+// are squared).
+struct Pair {
+    float hi = 0.0f, lo = 0.0f;
+};
+
+FR_D void pair_add(Pair& s, float x) {             // s += x (Knuth's two-sum)
+    const float t = __fadd_rn(s.hi, x), b = __fsub_rn(t, s.hi);
+    s.lo = __fadd_rn(s.lo, __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, b)), __fsub_rn(x, b)));
+    s.hi = t;
+}
+
+FR_D void pair_add_square(Pair& s, float w, float x) {     // s += w x^2
+    const float q = __fmul_rn(x, x), qe = __fmaf_rn(x, x, -q);
+    const float p = __fmul_rn(w, q), pe = __fmaf_rn(w, q, -p);
+    pair_add(s, p);
+    s.lo = __fadd_rn(s.lo, __fmaf_rn(w, qe, pe));
+}
+
+FR_D void pair_add_product(Pair& s, float w, float x) {    // s += w x
+    const float p = __fmul_rn(w, x);
+    pair_add(s, p);
+    s.lo = __fadd_rn(s.lo, __fmaf_rn(w, x, -p));
+}
+
+// The energy of texel t in FP64, for texels whose FP32 products overflow.
+__device__ __noinline__ double texel_energy64(const fr_opt_group& G, int C, int t) {
+    const int M = G.width;
+    const int row = t / M, col = t - row * M;
+    const float* X = G.x;
+    const float* x = X + (size_t)t * C;
+    double e = 0.0;
+    for (int c = 0; c < C; ++c) {
+        if (G.w_smooth != 0.0f) {
+            const int nb[4] = {t - 1, t + 1, t - M, t + M};
+            const bool in[4] = {col > 0, col < M - 1, row > 0, row < M - 1};
+            for (int k = 0; k < 4; ++k)
+                if (in[k]) {
+                    const double d = x[c] - X[(size_t)nb[k] * C + c];
+                    e += (double)G.w_smooth * d * d;
+                }
+        }
+        if (G.w_sym != 0.0f) e += (double)G.w_sym * fabsf(x[c] - X[((size_t)row * M + M - 1 - col) * C + c]);
+        if (G.w_box != 0.0f) {
+            const double lo = fminf(x[c], 0.0f), hi = fmaxf(x[c] - 1.0f, 0.0f);
+            e += (double)G.w_box * (lo * lo + hi * hi);
+        }
+    }
+    if (C == 3 && G.w_chroma != 0.0f && G.aux) {
+        const float* q = G.aux + (size_t)t * 3;
+        const float S = x[0] + x[1] + x[2] + 1e-6f, S0 = q[0] + q[1] + q[2] + 1e-6f;
+        for (int c = 0; c < 3; ++c) e += (double)G.w_chroma * fabsf(x[c] / S - q[c] / S0);
+    }
+    return e;
+}
+
+// Texture regularisers of texel t of a group of C channels: gradients g[C] of
+// its channels x[C], energies into e.  One thread takes a whole texel, so the
+// chromaticity's sums and quotients are formed once for its channels.
+template <int C, bool ENERGY>
+FR_D void texel_grad(const fr_opt_group& G, int t, const float (&x)[C], float (&g)[C], Pair& e) {
+    const int M = G.width;
+    const int row = t / M, col = t - row * M;
+    const float* X = G.x;
+    if (G.w_smooth != 0.0f) {                  // sum_i sum_{j in N4(i)} |X_j - X_i|^2: each ordered pair once here
+        const int nb[4] = {t - 1, t + 1, t - M, t + M};
+        const bool in[4] = {col > 0, col < M - 1, row > 0, row < M - 1};
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            float s = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (in[k]) {
+                    const float d = x[c] - X[(size_t)nb[k] * C + c];
+                    s += d;
+                    if (ENERGY) pair_add_square(e, G.w_smooth, d);
+                }
+            g[c] += 4.0f * G.w_smooth * s;
+        }
+    }
+    if (G.w_sym != 0.0f) {                     // sum |X(x) - X(flip x)|, flip: column -> M - 1 - column
+        const int fc = M - 1 - col;
+        if (fc != col) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const float d = x[c] - X[((size_t)row * M + fc) * C + c];
+                g[c] += 2.0f * G.w_sym * sgnf(d);
+                if (ENERGY) pair_add_product(e, G.w_sym, fabsf(d));
+            }
+        }
+    }
+    if (C == 3 && G.w_chroma != 0.0f && G.aux) {   // sum |kappa(X) - kappa(X0)|, kappa(c) = c / (sum c + 1e-6)
+        const float* q = G.aux + (size_t)t * 3;
+        const float S = x[0] + x[1] + x[2] + 1e-6f, S0 = q[0] + q[1] + q[2] + 1e-6f;
+        float kk[3], sg[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            kk[k] = x[k] / S;
+            const float d = kk[k] - q[k] / S0;
+            sg[k] = sgnf(d);
+            if (ENERGY) pair_add_product(e, G.w_chroma, fabsf(d));
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            float gc = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) gc += sg[k] * (((k == c) ? 1.0f : 0.0f) - kk[k]) / S;
+            g[c] += G.w_chroma * gc;
+        }
+    }
+    if (G.w_box != 0.0f) {                     // soft box [0, 1]
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const float lo = fminf(x[c], 0.0f), hi = fmaxf(x[c] - 1.0f, 0.0f);
+            g[c] += 2.0f * G.w_box * (lo + hi);
+            if (ENERGY && (lo != 0.0f || hi != 0.0f)) pair_add_square(e, G.w_box, lo + hi);   // one of them is 0
+        }
+    }
+}
+
+FR_D void update_moments(const GroupTable& T, const fr_opt_group& G, size_t i, float g) {
+    const float m = T.beta1 * G.m[i] + (1.0f - T.beta1) * g;
+    const float v = T.beta2 * G.v[i] + (1.0f - T.beta2) * g * g;
+    G.m[i] = m;
+    G.v[i] = v;
+}
+
+template <int C, bool ENERGY>
+FR_D void texel_moments(const GroupTable& T, const fr_opt_group& G, int t, Pair& e) {
+    float x[C], g[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        x[c] = G.x[(size_t)t * C + c];
+        g[c] = 0.0f;
+    }
+    texel_grad<C, ENERGY>(G, t, x, g, e);
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        const size_t i = (size_t)t * C + c;
+        update_moments(T, G, i, (G.g ? G.g[i] : 0.0f) + g[c]);
+    }
+}
+
 // Pass 1: gradient (render + regularisers) into m/v, reading x only; pass 2
 // applies the parameter update, so stencils read the pre-step values.
-FR_D int group_of_block(const GroupTable& T) {
-    int lo = 0, hi = T.n_groups - 1;          // last group whose start <= blockIdx.x
+FR_D int group_from(const int* start, int n_groups) {
+    int lo = 0, hi = n_groups - 1;            // last group whose start <= blockIdx.x
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (T.block_start[mid] <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
+        if (start[mid] <= (int)blockIdx.x) lo = mid; else hi = mid - 1;
     }
     return lo;
 }
 
+FR_D int group_of_block(const GroupTable& T) { return group_from(T.block_start, T.n_groups); }
+FR_D int group_of_apply_block(const GroupTable& T) { return group_from(T.apply_start, T.n_groups); }
+
+// A group's blocks cover its units: the texels of a texture group, the elements
+// of any other.
+template <bool ENERGY>
 __global__ void __launch_bounds__(ADAM_THREADS) k_adam_moments(GroupTable T, double* energy) {
     __shared__ double part[ADAM_THREADS / 32];
     const int gi = group_of_block(T);
     const fr_opt_group& G = T.g[gi];
     const int i = (blockIdx.x - T.block_start[gi]) * ADAM_THREADS + threadIdx.x;
     double e = 0.0;
-    if (i < G.n) {
-        const float x = G.x[i];
-        float g = G.g ? G.g[i] : 0.0f;
-        g += reg_grad(G, i, x, &e);
-        const float m = T.beta1 * G.m[i] + (1.0f - T.beta1) * g;
-        const float v = T.beta2 * G.v[i] + (1.0f - T.beta2) * g * g;
-        G.m[i] = m;
-        G.v[i] = v;
+    if (G.kind == FR_GROUP_TEX_RGB || G.kind == FR_GROUP_TEX_MONO) {   // block-uniform
+        Pair p;
+        if (G.kind == FR_GROUP_TEX_RGB) {
+            if (i < G.n / 3) texel_moments<3, ENERGY>(T, G, i, p);
+        } else if (i < G.n) {
+            texel_moments<1, ENERGY>(T, G, i, p);
+        }
+        if (ENERGY) {
+            double wide = 0.0;
+            if (!isfinite(p.hi + p.lo)) {          // (an overflow of its products, or not a finite texel)
+                wide = texel_energy64(G, G.kind == FR_GROUP_TEX_RGB ? 3 : 1, i);
+                p.hi = p.lo = 0.0f;
+            }
+            if (__any_sync(0xffffffffu, wide != 0.0))
+                for (int o = 16; o > 0; o >>= 1) wide += __shfl_xor_sync(0xffffffffu, wide, o);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float hi = __shfl_xor_sync(0xffffffffu, p.hi, o), lo = __shfl_xor_sync(0xffffffffu, p.lo, o);
+                pair_add(p, hi);
+                p.lo += lo;
+            }
+            if ((threadIdx.x & 31) == 0) e = (double)p.hi + (double)p.lo + wide;
+        }
+    } else {
+        if (i < G.n) {
+            const float x = G.x[i];
+            float g = G.g ? G.g[i] : 0.0f;
+            g += reg_grad(G, i, x, &e);
+            update_moments(T, G, i, g);
+        }
+        if (ENERGY)
+            for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
     }
-    if (energy) {
-        for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (ENERGY) {
         if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = e;
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -193,15 +330,33 @@ __global__ void __launch_bounds__(ADAM_THREADS) k_adam_moments(GroupTable T, dou
     }
 }
 
-__global__ void __launch_bounds__(ADAM_THREADS) k_adam_apply(GroupTable T) {
-    const int gi = group_of_block(T);
-    const fr_opt_group& G = T.g[gi];
-    const int i = (blockIdx.x - T.block_start[gi]) * ADAM_THREADS + threadIdx.x;
-    if (i >= G.n) return;
-    const float mh = G.m[i] / T.bc1[gi], vh = G.v[i] / T.bc2[gi];
-    float x = G.x[i] - G.lr * mh / (sqrtf(vh) + T.eps);
+// One element's update x - lr mh / (sqrt(vh) + eps), clamped.
+FR_D float adam_step(const fr_opt_group& G, const GroupTable& T, int gi, float x, float m, float v) {
+    const float mh = m / T.bc1[gi], vh = v / T.bc2[gi];
+    x = x - G.lr * mh / (sqrtf(vh) + T.eps);
     if (G.clamp_lo < G.clamp_hi) x = fminf(fmaxf(x, G.clamp_lo), G.clamp_hi);
-    G.x[i] = x;
+    return x;
+}
+
+// Four elements a thread, by 16-byte loads where the group's arrays allow.
+__global__ void __launch_bounds__(ADAM_THREADS) k_adam_apply(GroupTable T) {
+    const int gi = group_of_apply_block(T);
+    const fr_opt_group& G = T.g[gi];
+    const long i = ((long)(blockIdx.x - T.apply_start[gi]) * ADAM_THREADS + threadIdx.x) * 4;
+    if (i >= G.n) return;
+    const bool wide = ((reinterpret_cast<uintptr_t>(G.x) | reinterpret_cast<uintptr_t>(G.m) |
+                        reinterpret_cast<uintptr_t>(G.v)) & 15u) == 0;         // group-uniform
+    if (wide && i + 4 <= G.n) {
+        float4 x = *reinterpret_cast<const float4*>(G.x + i);
+        const float4 m = *reinterpret_cast<const float4*>(G.m + i), v = *reinterpret_cast<const float4*>(G.v + i);
+        x.x = adam_step(G, T, gi, x.x, m.x, v.x);
+        x.y = adam_step(G, T, gi, x.y, m.y, v.y);
+        x.z = adam_step(G, T, gi, x.z, m.z, v.z);
+        x.w = adam_step(G, T, gi, x.w, m.w, v.w);
+        *reinterpret_cast<float4*>(G.x + i) = x;
+        return;
+    }
+    for (long k = i; k < min(i + 4, (long)G.n); ++k) G.x[k] = adam_step(G, T, gi, G.x[k], G.m[k], G.v[k]);
 }
 
 }  // namespace
@@ -210,7 +365,7 @@ extern "C" fr_status fr_adam(const fr_opt_group* groups, int32_t n_groups, int32
                              float eps, double* reg_energy, void* stream) {
     if (!groups || n_groups < 1 || n_groups > FR_MAX_OPT_GROUPS || step < 1) return FR_EINVAL;
     GroupTable T;
-    int blocks = 0;
+    int blocks = 0, apply_blocks = 0;
     for (int k = 0; k < n_groups; ++k) {
         const fr_opt_group& G = groups[k];
         if (!G.x || !G.m || !G.v || G.n < 0) return FR_EINVAL;
@@ -224,9 +379,13 @@ extern "C" fr_status fr_adam(const fr_opt_group* groups, int32_t n_groups, int32
         T.bc1[k] = (float)(1.0 - pow((double)beta1, st_k));
         T.bc2[k] = (float)(1.0 - pow((double)beta2, st_k));
         T.block_start[k] = blocks;
-        blocks += (G.n + ADAM_THREADS - 1) / ADAM_THREADS;
+        T.apply_start[k] = apply_blocks;
+        const int units = G.kind == FR_GROUP_TEX_RGB ? G.n / 3 : G.n;
+        blocks += (units + ADAM_THREADS - 1) / ADAM_THREADS;
+        apply_blocks += (G.n + 4 * ADAM_THREADS - 1) / (4 * ADAM_THREADS);
     }
     T.block_start[n_groups] = blocks;
+    T.apply_start[n_groups] = apply_blocks;
     T.n_groups = n_groups;
     T.beta1 = beta1;
     T.beta2 = beta2;
@@ -234,8 +393,9 @@ extern "C" fr_status fr_adam(const fr_opt_group* groups, int32_t n_groups, int32
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (reg_energy) cudaMemsetAsync(reg_energy, 0, sizeof(double), st);
     if (blocks > 0) {
-        k_adam_moments<<<blocks, ADAM_THREADS, 0, st>>>(T, reg_energy);
-        k_adam_apply<<<blocks, ADAM_THREADS, 0, st>>>(T);
+        if (reg_energy) k_adam_moments<true><<<blocks, ADAM_THREADS, 0, st>>>(T, reg_energy);
+        else k_adam_moments<false><<<blocks, ADAM_THREADS, 0, st>>>(T, nullptr);
+        k_adam_apply<<<apply_blocks, ADAM_THREADS, 0, st>>>(T);
         fr_count_launches(2);
     }
     return cudaGetLastError() == cudaSuccess ? FR_OK : FR_ECUDA;
