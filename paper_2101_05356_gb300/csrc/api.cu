@@ -553,13 +553,11 @@ fr_status join_prep(fr_ctx* c, cudaStream_t st) {
 LossTable loss_table(fr_ctx* c, int n, const float* const* targets, double* const* losses, bool adjoint) {
     LossTable t;
     t.n = n;
-    t.max_px3 = 0;
     for (int k = 0; k < n; ++k) {
         const DevItem& it = c->h_items[k];
         const Slot& sl = c->slots[k];
         t.it[k] = LossItem{it.S.H, it.S.W, it.image, targets[k], losses[k], sl.sign, sl.loss_part, nullptr,
                            adjoint ? sl.adj_image : nullptr};
-        t.max_px3 = std::max(t.max_px3, it.S.H * it.S.W * 3);
     }
     return t;
 }

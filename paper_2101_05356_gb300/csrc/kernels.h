@@ -154,7 +154,6 @@ struct LossItem {
 };
 struct LossTable {
     int n;
-    int max_px3;
     LossItem it[FR_MAX_BATCH];
 };
 void launch_loss(const LossTable& t, cudaStream_t st);
