@@ -25,7 +25,7 @@ constexpr int LIN_GROUP = 8;
 // the G faces b of its group, with their coefficients staged in shared memory.
 // The basis terms are summed apart from the mean (they are much smaller), so
 // the large mean is rounded into the result once.
-template <int G>
+template <int G, int U>
 __global__ void __launch_bounds__(LIN_THREADS) k_linear(const float* __restrict__ mean,
                                                         const float* __restrict__ basis, int ld, int rows, int K,
                                                         LinearTable t) {
@@ -45,10 +45,9 @@ __global__ void __launch_bounds__(LIN_THREADS) k_linear(const float* __restrict_
     for (int b = 0; b < G; ++b) acc[b] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     const float4* bp = reinterpret_cast<const float4*>(basis) + i;
     // One face: U basis rows are loaded before any is summed, so that U loads
-    // are in flight per thread (its grid is small, 3N / 4 threads, a few warps
-    // per SM, and its time is the K / U dependent round trips to HBM).  A group
-    // keeps many warps per SM and unrolls by 8.  The sums run over k in order
-    // either way, so a face's result is the same in both.
+    // are in flight per thread (see the launcher for U).  A group keeps many
+    // warps per SM and unrolls by 8.  The sums run over k in order either way,
+    // so a face's result is the same in all.
     if constexpr (G > 1) {
 #pragma unroll 8
         for (int k = 0; k < K; ++k) {
@@ -60,7 +59,6 @@ __global__ void __launch_bounds__(LIN_THREADS) k_linear(const float* __restrict_
             }
         }
     } else {
-        constexpr int U = 36;
         for (int k0 = 0; k0 < K; k0 += U) {
             float4 bk[U];
 #pragma unroll
@@ -121,6 +119,29 @@ template <int NM>
 __device__ __forceinline__ int adj_model(const AdjLaunch& L, long x) {
     return (NM > 1 && x >= L.start[1]) ? 1 : 0;
 }
+// Sums of N values (a power of two <= 32) over the warp; value q is left in
+// lanes [q * 32 / N, (q + 1) * 32 / N).  Each step adds the lanes 16, 8, ... apart
+// and hands half of the values that are left to the other half of the lanes, so
+// every sum is the butterfly's, bit for bit, in N + log2(32 / N) - 1 shuffles
+// instead of 5 N.
+template <int N>
+__device__ __forceinline__ float warp_sums(float (&v)[N]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n >>= 1, o >>= 1) {
+        const bool high = lane & o;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float keep = high ? v[i + n] : v[i], send = high ? v[i] : v[i + n];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+#pragma unroll
+    for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
+}
+
 template <int G, int KG, int MIN_BLOCKS>
 __global__ void __launch_bounds__(LIN_THREADS, MIN_BLOCKS) k_linear_adj_part(const __grid_constant__ AdjLaunch L) {
     __shared__ float4 gs[G][ADJ_ROWS4];
@@ -157,33 +178,44 @@ __global__ void __launch_bounds__(LIN_THREADS, MIN_BLOCKS) k_linear_adj_part(con
         for (int q = 0; q < KG; ++q)
 #pragma unroll
             for (int b = 0; b < G; ++b) acc[q][b] = 0.0f;
+        if (nk == KG && lo + ADJ_ROWS4 <= rows4) {             // warp-uniform: no bounds to check
+            const float4* bp = reinterpret_cast<const float4*>(basis + (size_t)k0 * ld) + lo + lane;
 #pragma unroll 1
-        for (int r = lane; r < ADJ_ROWS4; r += 32) {
-            const int i = lo + r;
-            if (i >= rows4) break;
-            float4 bb[KG];
+            for (int r = 0; r < ADJ_ROWS4; r += 32) {
+                float4 bb[KG];
 #pragma unroll
-            for (int q = 0; q < KG; ++q)
-                bb[q] = q < nk ? __ldg(reinterpret_cast<const float4*>(basis + (size_t)(k0 + q) * ld) + i)
-                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                for (int q = 0; q < KG; ++q) bb[q] = __ldg(bp + (size_t)q * (ld / 4) + r);
 #pragma unroll
-            for (int b = 0; b < G; ++b) {
-                const float4 gg = gs[b][r];
+                for (int b = 0; b < G; ++b) {
+                    const float4 gg = gs[b][r + lane];
+#pragma unroll
+                    for (int q = 0; q < KG; ++q)
+                        acc[q][b] += bb[q].x * gg.x + bb[q].y * gg.y + bb[q].z * gg.z + bb[q].w * gg.w;
+                }
+            }
+        } else {
+#pragma unroll 1
+            for (int r = lane; r < ADJ_ROWS4; r += 32) {
+                const int i = lo + r;
+                if (i >= rows4) break;
+                float4 bb[KG];
 #pragma unroll
                 for (int q = 0; q < KG; ++q)
-                    acc[q][b] += bb[q].x * gg.x + bb[q].y * gg.y + bb[q].z * gg.z + bb[q].w * gg.w;
+                    bb[q] = q < nk ? __ldg(reinterpret_cast<const float4*>(basis + (size_t)(k0 + q) * ld) + i)
+                                   : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+                for (int b = 0; b < G; ++b) {
+                    const float4 gg = gs[b][r];
+#pragma unroll
+                    for (int q = 0; q < KG; ++q)
+                        acc[q][b] += bb[q].x * gg.x + bb[q].y * gg.y + bb[q].z * gg.z + bb[q].w * gg.w;
+                }
             }
         }
-        // the butterfly leaves the same sum, bitwise, on every lane
-#pragma unroll
-        for (int q = 0; q < KG; ++q)
-#pragma unroll
-            for (int b = 0; b < G; ++b) {
-                float v = acc[q][b];
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (lane == ((q * G + b) & 31) && q < nk && b < nb_)
-                    part[((size_t)chunk * t.n + b0 + b) * K + k0 + q] = (double)v;
-            }
+        const float v = warp_sums<KG * G>(reinterpret_cast<float(&)[KG * G]>(acc));
+        constexpr int W = 32 / (KG * G);
+        const int q = lane / W / G, b = lane / W % G;
+        if (lane % W == 0 && q < nk && b < nb_) part[((size_t)chunk * t.n + b0 + b) * K + k0 + q] = (double)v;
     }
 }
 
@@ -193,8 +225,12 @@ __global__ void __launch_bounds__(LIN_THREADS, MIN_BLOCKS) k_linear_adj_part(con
 // same butterfly), so the partials are bitwise those of the face in a batch.
 // The gradient is read from global memory (consecutive warps share a chunk, so
 // it is an L1 hit after the first), which leaves no shared staging to balance
-// over the block's warps.
-template <int KG>
+// over the block's warps.  RB rows' loads are in flight before they are summed,
+// in the same order.  Bound by HBM: 510 MB for both 512 x 512 albedos at K = 80,
+// 75 us; measured 87 us with the second pass, against 119 us with eight columns
+// a warp, one row in flight and five shuffles a sum (four columns: 88 us).
+constexpr int ONE_K = 2, ONE_ROWS = 4;
+template <int KG, int RB>
 __global__ void __launch_bounds__(LIN_THREADS) k_linear_adj_one(const __grid_constant__ AdjLaunch L) {
     const int lane = threadIdx.x & 31;
     const long gitem = (long)blockIdx.x * (LIN_THREADS / 32) + (threadIdx.x >> 5);
@@ -212,32 +248,49 @@ __global__ void __launch_bounds__(LIN_THREADS) k_linear_adj_one(const __grid_con
     float acc[KG];
 #pragma unroll
     for (int q = 0; q < KG; ++q) acc[q] = 0.0f;
+    if (nk == KG && 4 * (lo + ADJ_ROWS4) <= rows) {            // warp-uniform
+        const float4* bp = reinterpret_cast<const float4*>(basis + (size_t)k0 * ld) + lo + lane;
+        const float4* gp = reinterpret_cast<const float4*>(g) + lo + lane;
 #pragma unroll 1
-    for (int r = lane; r < ADJ_ROWS4; r += 32) {
-        const int i = lo + r, e = 4 * i;
-        if (i >= rows4) break;
-        float4 gg = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (e + 4 <= rows) {
-            gg = *reinterpret_cast<const float4*>(g + e);
-        } else {                                       // ragged tail
-            gg.x = g[e];
-            if (e + 1 < rows) gg.y = g[e + 1];
-            if (e + 2 < rows) gg.z = g[e + 2];
+        for (int r = 0; r < ADJ_ROWS4; r += 32 * RB) {
+            float4 bb[RB][KG], gg[RB];
+#pragma unroll
+            for (int j = 0; j < RB; ++j) {
+                gg[j] = gp[r + 32 * j];
+#pragma unroll
+                for (int q = 0; q < KG; ++q) bb[j][q] = __ldg(bp + (size_t)q * (ld / 4) + r + 32 * j);
+            }
+#pragma unroll
+            for (int j = 0; j < RB; ++j)
+#pragma unroll
+                for (int q = 0; q < KG; ++q)
+                    acc[q] += bb[j][q].x * gg[j].x + bb[j][q].y * gg[j].y + bb[j][q].z * gg[j].z + bb[j][q].w * gg[j].w;
         }
-        float4 bb[KG];
+    } else {
+#pragma unroll 1
+        for (int r = lane; r < ADJ_ROWS4; r += 32) {
+            const int i = lo + r, e = 4 * i;
+            if (i >= rows4) break;
+            float4 gg = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (e + 4 <= rows) {
+                gg = *reinterpret_cast<const float4*>(g + e);
+            } else {                                       // ragged tail
+                gg.x = g[e];
+                if (e + 1 < rows) gg.y = g[e + 1];
+                if (e + 2 < rows) gg.z = g[e + 2];
+            }
+            float4 bb[KG];
 #pragma unroll
-        for (int q = 0; q < KG; ++q)
-            bb[q] = q < nk ? __ldg(reinterpret_cast<const float4*>(basis + (size_t)(k0 + q) * ld) + i)
-                           : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            for (int q = 0; q < KG; ++q)
+                bb[q] = q < nk ? __ldg(reinterpret_cast<const float4*>(basis + (size_t)(k0 + q) * ld) + i)
+                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-        for (int q = 0; q < KG; ++q) acc[q] += bb[q].x * gg.x + bb[q].y * gg.y + bb[q].z * gg.z + bb[q].w * gg.w;
+            for (int q = 0; q < KG; ++q) acc[q] += bb[q].x * gg.x + bb[q].y * gg.y + bb[q].z * gg.z + bb[q].w * gg.w;
+        }
     }
-#pragma unroll
-    for (int q = 0; q < KG; ++q) {
-        float v = acc[q];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == (q & 31) && q < nk) part[((size_t)chunk * t.n) * K + k0 + q] = (double)v;
-    }
+    const float v = warp_sums<KG>(acc);
+    constexpr int W = 32 / KG;
+    if (lane % W == 0 && lane / W < nk) part[((size_t)chunk * t.n) * K + k0 + lane / W] = (double)v;
 }
 
 // Adjoint, second pass: g_coef_b[k] += the sum of the chunk partials.  Block
@@ -270,6 +323,17 @@ __global__ void __launch_bounds__(FIN_THREADS) k_linear_adj_finish(const __grid_
 
 int nb(long n, int t) { return (int)((n + t - 1) / t); }
 
+int sm_count() {
+    static int sms = 0;
+    if (!sms) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (sms <= 0) sms = 1;
+    }
+    return sms;
+}
+
 }  // namespace
 
 int linear_adj_chunks(int rows) { return std::max(1, nb((rows + 3) / 4, ADJ_ROWS4)); }
@@ -282,10 +346,20 @@ void launch_linear(const float* mean, const float* basis, int ld, int rows, int 
     // the columns over several threads per row would keep more loads in flight,
     // but its sums would differ from the batched kernel's in the last bits, and
     // a face must render bitwise the same alone and in a batch.)
-    if (t.n == 1)
-        k_linear<1><<<nb((rows + 3) / 4, LIN_THREADS / 4), LIN_THREADS / 4, 0, st>>>(mean, basis, ld, rows, K, t);
-    else
-        k_linear<LIN_GROUP><<<grid, LIN_THREADS, 0, st>>>(mean, basis, ld, rows, K, t);
+    // With at most the four blocks per SM that 36 loads in flight leave room for,
+    // the time is the K / 36 round trips to HBM (the 107,127-row shape model); with
+    // more, 12 loads leave room for three times the warps, whose loads overlap
+    // each other's sums and fill the last wave (both 512 x 512 albedos: 36 loads
+    // 0.110 ms, 20: 0.095, 16: 0.087, 12: 0.082, 8: 0.086; HBM alone 0.076 ms).
+    if (t.n == 1) {
+        const int blocks = nb((rows + 3) / 4, LIN_THREADS / 4);
+        if (blocks <= 4 * sm_count())
+            k_linear<1, 36><<<blocks, LIN_THREADS / 4, 0, st>>>(mean, basis, ld, rows, K, t);
+        else
+            k_linear<1, 12><<<blocks, LIN_THREADS / 4, 0, st>>>(mean, basis, ld, rows, K, t);
+    } else {
+        k_linear<LIN_GROUP, 8><<<grid, LIN_THREADS, 0, st>>>(mean, basis, ld, rows, K, t);
+    }
     fr_count_launches(1);
 }
 
@@ -308,36 +382,31 @@ void launch_linear_adjoint(const LinearAdjModel* models, int n_models, cudaStrea
         kmax = std::max(kmax, md.K);
     }
     if (L.n_models == 0) return;
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 1;
-    }
+    const int sms = sm_count();
     const int n_groups = nb(n, LIN_GROUP);
     L.start[0] = 0;
     if (n == 1) {
         // one launch per model: the model's table is then constant in the kernel
-        // (48 registers; selecting the model per warp took 57 and measured slower)
         for (int m = 0; m < L.n_models; ++m) {
             AdjLaunch L1 = L;
             L1.n_models = 1;
             L1.basis[0] = L.basis[m]; L1.ld[0] = L.ld[m]; L1.rows[0] = L.rows[m]; L1.K[0] = L.K[m];
             L1.chunks[0] = L.chunks[m]; L1.part[0] = L.part[m]; L1.t[0] = L.t[m];
             L1.start[0] = 0;
-            L1.start[1] = L.chunks[m] * nb(L.K[m], 8);
-            k_linear_adj_one<8><<<nb(L1.start[1], LIN_THREADS / 32), LIN_THREADS, 0, st>>>(L1);
+            L1.start[1] = L.chunks[m] * nb(L.K[m], ONE_K);
+            k_linear_adj_one<ONE_K, ONE_ROWS><<<nb(L1.start[1], LIN_THREADS / 32), LIN_THREADS, 0, st>>>(L1);
         }
         fr_count_launches(L.n_models - 1);
     } else {
         for (int m = 0; m < L.n_models; ++m) L.start[m + 1] = L.start[m] + L.chunks[m];
         // split the columns over grid.z until about eight blocks per SM are in flight
-        // (measured on GB300, albedo batch 8, both models: two columns per warp at six
-        // blocks per SM (40 registers) 0.163 ms; at five 0.183-0.189 ms, at seven or
-        // eight (spilling) 0.228 ms, four columns at four 0.185 ms)
+        // (measured on GB300, albedo batch 8, both models, 1,536 chunks: 0.125 ms; with
+        // the columns split over 2, 3, 4, 5 blocks 0.132, 0.138, 0.144, 0.155 ms.  Two
+        // columns per warp at six blocks per SM (40 registers); four columns at four
+        // blocks 0.126, at five, spilling, 0.196 ms; two or four rows' loads in flight
+        // at the fewer blocks they leave 0.16-0.18 ms)
         const int most = nb(nb(kmax, 2), LIN_THREADS / 32);
-        const int z = std::max(1, std::min(most, nb(8L * sms, (long)L.start[L.n_models] * n_groups)));
+                const int z = std::max(1, std::min(most, nb(8L * sms, (long)L.start[L.n_models] * n_groups)));
         k_linear_adj_part<LIN_GROUP, 2, 6><<<dim3(L.start[L.n_models], n_groups, z), LIN_THREADS, 0, st>>>(L);
     }
     k_linear_adj_finish<<<dim3(nb(kmax, FIN_K), n, L.n_models), FIN_THREADS, 0, st>>>(L);
