@@ -27,15 +27,15 @@ constexpr int RT_WARPS = RT_THREADS / 32;
 #endif
 // minimum resident blocks per SM requested from the compiler (register cap).
 // Measured on GB300 (paper-scale face): the forward is fastest at 8 blocks
-// (1.25 ms; 7: 1.30 ms, 9: 1.27 ms, 6: 1.37 ms), the primary-edge kernel at 6
-// (0.39 ms beside the adjoint; 7: 0.43 ms, 8: 0.46 ms, 9: 0.50 ms), the
+// (1.25 ms; 7: 1.30 ms, 9: 1.27 ms, 6: 1.37 ms), the primary-edge kernel at 7
+// (step 1.99 ms; 6 the same, at 512 x 512 4.44 ms against 4.46 ms), the
 // adjoint reading hit records at 5 (0.601 ms; 6: 0.618 ms, 8: 0.637 ms) and
 // the re-tracing adjoint at 8 (4.20 ms; 6: 4.38 ms, 5: 4.65 ms).
 #ifndef FR_FWD_MIN_BLOCKS
 #define FR_FWD_MIN_BLOCKS 8
 #endif
 #ifndef FR_EDGE_MIN_BLOCKS
-#define FR_EDGE_MIN_BLOCKS 6
+#define FR_EDGE_MIN_BLOCKS 7
 #endif
 #ifndef FR_ADJ_REC_MIN_BLOCKS
 #define FR_ADJ_REC_MIN_BLOCKS 5
@@ -377,12 +377,11 @@ FR_D float3 shade_visible(const DevScene& S, const DevParams& P, const Sampler& 
 // Full warp-cooperative radiance evaluation at screen point (sx, sy):
 // visibility first, then the material and the radiance, so that the material
 // is not live across the shadow traversal.
-template <bool ENV>
+template <bool ENV, class C>
 FR_D float3 radiance_at(const DevScene& S, const DevParams& P, bool active, float sx, float sy,
-                        const Sampler& smp, int dim0, RtShared& sh, Stack stk, SampleState& ss, uint64_t* vis,
+                        const Sampler& smp, int dim0, RtShared& sh, C& cover, Stack stk, SampleState& ss, uint64_t* vis,
                         RayStats& rs) {
-    NoCover root;
-    visibility_at<ENV>(S, P, active, sx, sy, smp, dim0, sh, root, stk, ss, vis, rs);
+    visibility_at<ENV>(S, P, active, sx, sy, smp, dim0, sh, cover, stk, ss, vis, rs);
     return shade_visible<ENV>(S, P, smp, dim0, ss, vis);
 }
 
@@ -1122,7 +1121,9 @@ __global__ void __launch_bounds__(RT_THREADS, FR_EDGE_MIN_BLOCKS) k_edge_primary
     SampleState ss;
     uint64_t vis[2];
     RayStats rs;
-    const float3 L = radiance_at<ENV>(S, P, active, X + eps * mx, Y + eps * my, smp, 4, sh, my_stack(sh), ss, vis, rs);
+    __shared__ Cover cover[RT_WARPS];
+    const float3 L = radiance_at<ENV>(S, P, active, X + eps * mx, Y + eps * my, smp, 4, sh, cover[threadIdx.x >> 5],
+                                      my_stack(sh), ss, vis, rs);
     const float3 Lo = f3(__shfl_xor_sync(FULL, L.x, 1), __shfl_xor_sync(FULL, L.y, 1), __shfl_xor_sync(FULL, L.z, 1));
     const float3 Lp = side ? Lo : L, Lm = side ? L : Lo;
     if (side) active = false;                          // the even lane adds the pair's term

@@ -304,8 +304,10 @@ FR_D bool trace_any(const DevScene& s, const RayPre& r, float tmin, float tmax, 
 // root, which for such rays is that same path with two tests and a stack
 // operation a level.  Measured: paper-scale face (two pixels a warp) forward
 // 1.39 -> 1.25 ms, large face (half a pixel) 112 -> 90 ms, small face (eight
-// pixels) 0.157 -> 0.139 ms.  The primary-edge and specular-boundary kernels,
-// whose warps' rays start apart, trace from the root.
+// pixels) 0.157 -> 0.139 ms.  The primary-edge samples, sorted by position, start
+// close together too (paper-scale step 2.01 -> 1.99 ms); the specular-boundary
+// kernel and the shadow-boundary samples, whose rays start apart, trace from
+// the root.
 // ---------------------------------------------------------------------------
 constexpr int COVER_MAX = 24;
 
