@@ -71,6 +71,7 @@ struct LinearModel {
 struct fr_ctx {
     fr_config cfg{};
     int max_batch = 1;
+    int sms = 1;
     int N = 0, T = 0, K = 0, NL = 0, E = 0, ld = 0;   // ld = shape.ld
     bool have_mesh = false, have_lights = false;
     bool poisoned = false;                     // a device wait gave up unsafely: refuse further work
@@ -285,10 +286,10 @@ DevItem make_item(const fr_ctx* c, int k, const ItemArgs& a) {
     return it;
 }
 
-// Blocks of a launch over camera samples [q0, q0 + cap) of each item, for the
-// items `take` accepts (the others get no blocks).
+// Blocks of a launch over camera samples [q0, q0 + cap) of each item, `per`
+// samples a block, for the items `take` accepts (the others get no blocks).
 template <class F>
-BlockMap tile_map(const fr_ctx* c, int n, long q0, long cap, F take) {
+BlockMap tile_map(const fr_ctx* c, int n, long q0, long cap, F take, int per = 128) {
     BlockMap m;
     m.n = n;
     int b = 0;
@@ -296,13 +297,13 @@ BlockMap tile_map(const fr_ctx* c, int n, long q0, long cap, F take) {
         const DevScene& s = c->h_items[k].S;
         m.block0[k] = b;
         const long left = (long)s.W * s.H * s.spp - q0;
-        if (take(c->h_items[k]) && left > 0) b += (int)((std::min(left, cap) + 127) / 128);
+        if (take(c->h_items[k]) && left > 0) b += (int)((std::min(left, cap) + per - 1) / per);
     }
     m.block0[n] = b;
     return m;
 }
 
-BlockMap map_of(const fr_ctx* c, int n, bool edges) {
+BlockMap map_of(const fr_ctx* c, int n, bool edges, int per = 128) {
     BlockMap m;
     m.n = n;
     int b = 0;
@@ -311,10 +312,32 @@ BlockMap map_of(const fr_ctx* c, int n, bool edges) {
         m.block0[k] = b;
         // primary-edge samples take two threads each (one per side of the edge)
         long work = (long)s.W * s.H * (edges ? ((s.flags & FR_FLAG_NO_PRIMARY_EDGE) ? 0 : 2 * s.edge_spp) : s.spp);
-        b += (int)((work + 127) / 128);
+        b += (int)((work + per - 1) / per);
     }
     m.block0[n] = b;
     return m;
+}
+
+// Few blocks: their warps then share the shadow rays of 32 samples instead of
+// holding 32 samples each, so that four times the warps cover the latency of
+// the walks, and the longest chain of walks is a quarter as long (they trace the
+// camera rays four times).  The lines, in blocks per SM of the unsplit launch,
+// lie where both sides were measured equal: forward at 8 lights 128 blocks 0.141
+// -> 0.098 ms, 512 blocks 0.137 -> 0.113, 800 blocks 0.143 -> 0.133, 1,280 blocks
+// 0.172 -> 0.193; at 40 lights 1,024 blocks 0.541 -> 0.406, 1,600 blocks 0.61 ->
+// 0.53, 1,967 blocks 0.65 -> 0.71; 64 environment blocks, 1,024 blocks, forward
+// and its records-only pass 2.88 -> 2.13 ms.  Primary edges
+// (the step's time): 64 blocks at 40 lights 0.87 -> 0.53 ms with the forward's,
+// 256 blocks at 40 lights 0.97 -> 0.85, 640 blocks at 8 lights 0.49 -> 0.52,
+// 1,024 blocks at 40 lights 1.99 -> 2.08.
+constexpr int SPLIT_FORWARD = 8, SPLIT_FORWARD_MANY = 11, SPLIT_MANY_LIGHTS = 32, SPLIT_EDGE = 4;
+
+int split_forward(const fr_ctx* c) { return c->NL >= SPLIT_MANY_LIGHTS ? SPLIT_FORWARD_MANY : SPLIT_FORWARD; }
+
+bool split_lights(const fr_ctx* c, int n, const BlockMap& unsplit, int per_sm) {
+    for (int k = 0; k < n; ++k)
+        if (c->h_items[k].S.spp > 32) return false;
+    return unsplit.block0[unsplit.n] <= per_sm * c->sms;
 }
 
 // One block per scanline of the specular-boundary term for each item that has
@@ -439,7 +462,10 @@ fr_status forward_pass(fr_ctx* c, int n, cudaStream_t st) {
         // sums are added onto zero (exact in either order)
         if (it.S.spp > 128) CK(c, cudaMemsetAsync(it.image, 0, sizeof(float) * 3 * (size_t)it.S.W * it.S.H, st));
     }
-    launch_forward(c->d_items, map_of(c, n, false), c->env_size > 0, 0, false, st);
+    BlockMap map = map_of(c, n, false);
+    const bool split = split_lights(c, n, map, split_forward(c));
+    if (split) map = map_of(c, n, false, 32);
+    launch_forward(c->d_items, map, c->env_size > 0, split, 0, false, st);
     return FR_OK;
 }
 
@@ -471,7 +497,10 @@ fr_status adjoint_main(fr_ctx* c, int n, cudaStream_t st) {
     mark(c, 4, st);
     CK(c, cudaEventRecord(c->fork_ev, st));
     CK(c, cudaStreamWaitEvent(c->side, c->fork_ev, 0));
-    launch_edge_primary(c->d_items, map_of(c, n, true), c->env_size > 0, c->side);
+    BlockMap emap = map_of(c, n, true);
+    const bool esplit = split_lights(c, n, emap, SPLIT_EDGE);
+    if (esplit) emap = map_of(c, n, true, 32);
+    launch_edge_primary(c->d_items, emap, c->env_size > 0, esplit, c->side);
     launch_edge_specular(c->d_items, spec_map(c, n), c->env_size > 0, c->side);
     CK(c, cudaEventRecord(c->join_ev, c->side));
     bool all_full = true, any_retrace = false, any_stage = false;
@@ -500,9 +529,11 @@ fr_status adjoint_main(fr_ctx* c, int n, cudaStream_t st) {
         }
         for (long t = n_tiles - 1; t >= 0; --t) {
             const long q0 = t * cap;
-            launch_forward(c->d_items,
-                           tile_map(c, n, q0, cap, [q0](const DevItem& it) { return !it.rec_full && it.rec_from != q0; }),
-                           env, q0, true, st);
+            const auto lacks = [q0](const DevItem& it) { return !it.rec_full && it.rec_from != q0; };
+            BlockMap map = tile_map(c, n, q0, cap, lacks);
+            const bool split = split_lights(c, n, map, split_forward(c));
+            if (split) map = tile_map(c, n, q0, cap, lacks, 32);
+            launch_forward(c->d_items, map, env, split, q0, true, st);
             launch_adjoint(c->d_items, tile_map(c, n, q0, cap, [](const DevItem&) { return true; }), c->NL, true,
                            any_stage, env, q0, st);
         }
@@ -683,6 +714,10 @@ fr_status fr_create(fr_ctx** out, const fr_config* cfg) {
     fr_ctx* c = new fr_ctx();
     c->cfg = *cfg;
     c->max_batch = std::max(1, cfg->max_batch);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || c->sms < 1)
+        c->sms = 1;
     c->slots.resize(c->max_batch);
     c->h_items.resize(FR_MAX_BATCH);
     const size_t px = (size_t)cfg->width * cfg->height * 3;

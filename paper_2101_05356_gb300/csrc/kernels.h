@@ -127,12 +127,12 @@ void launch_bvh_check(const DevItem* items, int T, int* out, cudaStream_t st);
 // render.cu
 // the ray kernels process camera samples [q0, q0 + count) of each item, count
 // from the block map; records_only: the adjoint's records of that tile only
-void launch_forward(const DevItem* items, const BlockMap& map, bool env, long q0, bool records_only,
+void launch_forward(const DevItem* items, const BlockMap& map, bool env, bool split, long q0, bool records_only,
                     cudaStream_t st);
 void launch_adjoint(const DevItem* items, const BlockMap& map, int NL, bool all_recorded, bool any_stage, bool env,
                     long q0, cudaStream_t st);
 void launch_edge_order(const DevItem* items, int n, long max_edge, cudaStream_t st);
-void launch_edge_primary(const DevItem* items, const BlockMap& map, bool env, cudaStream_t st);
+void launch_edge_primary(const DevItem* items, const BlockMap& map, bool env, bool split, cudaStream_t st);
 void launch_classify(const DevItem* items, int n, int E, int NL, int T, cudaStream_t st);
 void launch_spec_candidates(const DevItem* items, int n, int T, const BlockMap& map, cudaStream_t st);
 void launch_edge_specular(const DevItem* items, const BlockMap& map, bool env, cudaStream_t st);

@@ -187,9 +187,11 @@ FR_D void drain(const DevScene& S, WarpQueue& q, const C& cover, int head, int n
 // Warp-cooperative shadow visibility for the lights [j0, j0 + 64): bit j - j0
 // is set when the shadow ray to this lane's light-j sample is traced and
 // unoccluded.  All 32 lanes must call this together.
-template <bool ENV, class C>
+// SPLIT > 1: this warp takes only the lights whose sample's Philox block is
+// `sub` modulo SPLIT (two lights share a block).
+template <bool ENV, int SPLIT = 1, class C>
 FR_D uint64_t shadow_mask(const DevScene& S, const SampleState& ss, const Sampler& smp, int dim0,
-                          WarpQueue& q, const C& cover, Stack st, RayStats& rs, int j0) {
+                          WarpQueue& q, const C& cover, Stack st, RayStats& rs, int j0, int sub = 0) {
     const int lane = threadIdx.x & 31;
     q.vis[lane] = 0ull;
     __syncwarp();
@@ -200,6 +202,7 @@ FR_D uint64_t shadow_mask(const DevScene& S, const SampleState& ss, const Sample
     // light by light, then (j = j1) what is left in the ring: one place that
     // traces, so the kernel holds its code once
     for (int j = j0; j <= j1; ++j) {
+        if (SPLIT > 1 && j < j1 && ((dim0 + 2 * j) >> 2) % SPLIT != sub) continue;
         bool need = false;
         float3 z = f3(0.0f, 0.0f, 0.0f);
         const bool distant = ENV && j < j1 && S.lights[j].type == FR_LIGHT_ENV_D;      // warp-uniform
@@ -353,15 +356,32 @@ FR_D void make_cover(const DevScene& S, const SampleState& ss, Cover& c) {
     build_cover(S, c, __ballot_sync(FULL, ss.hit && ss.lit), ss.slot);
 }
 
-template <bool ENV, class C>
+// SPLIT > 1: the block's SPLIT warps hold the same samples; each traces the
+// camera rays and its share of the shadow rays, and all return every bit.
+template <bool ENV, int SPLIT, class C>
 FR_D void visibility_at(const DevScene& S, const DevParams& P, bool active, float sx, float sy,
                         const Sampler& smp, int dim0, RtShared& sh, C& cover, Stack stk, SampleState& ss,
                         uint64_t* vis, RayStats& rs) {
+    static_assert(SPLIT == 1 || SPLIT == RT_WARPS, "the block's warps share its samples");
+    const int warp = threadIdx.x >> 5;
     primary_state<true, false>(S, P, active, sx, sy, stk, ss, rs);
+    if (SPLIT > 1 && warp > 0) rs = RayStats();              // the first warp counts the camera rays
     make_cover(S, ss, cover);
     vis[0] = vis[1] = 0ull;
     for (int j0 = 0; j0 < max(S.NL, 1); j0 += 64)            // lights in chunks of 64 (warp-uniform)
-        vis[j0 >> 6] = shadow_mask<ENV>(S, ss, smp, dim0, sh.wq[threadIdx.x >> 5], cover, stk, rs, j0);
+        vis[j0 >> 6] = shadow_mask<ENV, SPLIT>(S, ss, smp, dim0, sh.wq[warp], cover, stk, rs, j0, warp);
+    if (SPLIT > 1) {
+        const int lane = threadIdx.x & 31;
+        uint64_t* mine = reinterpret_cast<uint64_t*>(sh.wq[warp].job);        // the warp's jobs are done
+        mine[lane] = vis[0];
+        mine[32 + lane] = vis[1];
+        __syncthreads();
+        for (int w = 0; w < SPLIT; ++w) {
+            const uint64_t* o = reinterpret_cast<const uint64_t*>(sh.wq[w].job);
+            vis[0] |= o[lane];
+            vis[1] |= o[32 + lane];
+        }
+    }
 }
 
 // Radiance of a sample whose visibility is known: the material, then the lights.
@@ -377,11 +397,11 @@ FR_D float3 shade_visible(const DevScene& S, const DevParams& P, const Sampler& 
 // Full warp-cooperative radiance evaluation at screen point (sx, sy):
 // visibility first, then the material and the radiance, so that the material
 // is not live across the shadow traversal.
-template <bool ENV, class C>
+template <bool ENV, int SPLIT, class C>
 FR_D float3 radiance_at(const DevScene& S, const DevParams& P, bool active, float sx, float sy,
                         const Sampler& smp, int dim0, RtShared& sh, C& cover, Stack stk, SampleState& ss, uint64_t* vis,
                         RayStats& rs) {
-    visibility_at<ENV>(S, P, active, sx, sy, smp, dim0, sh, cover, stk, ss, vis, rs);
+    visibility_at<ENV, SPLIT>(S, P, active, sx, sy, smp, dim0, sh, cover, stk, ss, vis, rs);
     return shade_visible<ENV>(S, P, smp, dim0, ss, vis);
 }
 
@@ -425,7 +445,10 @@ FR_D void store_vis(const DevScene& S, uint64_t* rec_vis, long i, const uint64_t
 // nothing.  Otherwise: the forward render, writing the records of samples
 // q >= it.rec_from at q - it.rec_from (the whole image when it fits the
 // record buffer, else its last tile; it.rec_from < 0: none).
-template <bool ENV>
+//
+// SPLIT > 1 (launches of few blocks, at most 32 samples a pixel): a block takes
+// 32 samples, its warps their shadow rays between them, the first warp the rest.
+template <bool ENV, int SPLIT>
 __global__ void __launch_bounds__(RT_THREADS, FR_FWD_MIN_BLOCKS) k_forward(const DevItem* items, BlockMap map,
                                                                            long q0, int records_only) {
     __shared__ RtShared sh;
@@ -439,7 +462,8 @@ __global__ void __launch_bounds__(RT_THREADS, FR_FWD_MIN_BLOCKS) k_forward(const
     uint64_t* mask_rec = it.mask_rec;
     const uint32_t iteration = it.iteration, face = it.face;
     const long total = (long)S.W * S.H * S.spp;
-    const long ql = (long)(blockIdx.x - map.block0[item]) * RT_THREADS + threadIdx.x;
+    const long ql = SPLIT > 1 ? (long)(blockIdx.x - map.block0[item]) * 32 + (threadIdx.x & 31)
+                              : (long)(blockIdx.x - map.block0[item]) * RT_THREADS + threadIdx.x;
     const long q = q0 + ql;
     const bool valid = q < total;
     const int pixel = valid ? (int)(q / S.spp) : 0;
@@ -450,8 +474,12 @@ __global__ void __launch_bounds__(RT_THREADS, FR_FWD_MIN_BLOCKS) k_forward(const
     uint64_t vis[2];
     RayStats rs;
     __shared__ Cover cover[RT_WARPS];
-    visibility_at<ENV>(S, P, valid, (float)(pixel % S.W) + jit.x, (float)(pixel / S.W) + jit.y, smp, 2, sh,
-                       cover[threadIdx.x >> 5], my_stack(sh), ss, vis, rs);
+    visibility_at<ENV, SPLIT>(S, P, valid, (float)(pixel % S.W) + jit.x, (float)(pixel / S.W) + jit.y, smp, 2, sh,
+                              cover[threadIdx.x >> 5], my_stack(sh), ss, vis, rs);
+    if (SPLIT > 1 && threadIdx.x >= 32) {
+        flush_stats(S.counters + (records_only ? 3 : 0), rs);
+        return;
+    }
     if (records_only) {                                 // launch-uniform
         flush_stats(S.counters + 3, rs);                // the adjoint's rays
         if (valid) {
@@ -480,7 +508,7 @@ __global__ void __launch_bounds__(RT_THREADS, FR_FWD_MIN_BLOCKS) k_forward(const
     const int width = S.spp < 32 ? S.spp : 32;
     const float rx = group_sum(Lo.x, width), ry = group_sum(Lo.y, width), rz = group_sum(Lo.z, width);
     const float inv = 1.0f / (float)S.spp;
-    if (S.spp <= 32) {
+    if (SPLIT > 1 || S.spp <= 32) {
         if (valid && (s % width) == 0) {
             float* px = image + 3 * (size_t)pixel;
             px[0] = rx * inv; px[1] = ry * inv; px[2] = rz * inv;
@@ -1058,7 +1086,8 @@ __global__ void __launch_bounds__(EDGE_SORT_THREADS) k_edge_order(const DevItem*
 // ---------------------------------------------------------------------------
 // primary-visibility boundary term: edge samples in screen space
 // ---------------------------------------------------------------------------
-template <bool ENV>
+// SPLIT > 1: as in k_forward.
+template <bool ENV, int SPLIT>
 __global__ void __launch_bounds__(RT_THREADS, FR_EDGE_MIN_BLOCKS) k_edge_primary(const DevItem* items, BlockMap map) {
     __shared__ RtShared sh;
     FR_STACK_DECL
@@ -1075,7 +1104,8 @@ __global__ void __launch_bounds__(RT_THREADS, FR_EDGE_MIN_BLOCKS) k_edge_primary
     // two lanes per edge sample: the even one evaluates the radiance on the
     // + side of the edge, the odd one on the - side (twice the warps of one
     // lane doing both in turn; the same samples and the same arithmetic)
-    const long t0 = (long)(blockIdx.x - map.block0[item]) * RT_THREADS + threadIdx.x;
+    const long t0 = SPLIT > 1 ? (long)(blockIdx.x - map.block0[item]) * 32 + (threadIdx.x & 31)
+                              : (long)(blockIdx.x - map.block0[item]) * RT_THREADS + threadIdx.x;
     const long e0 = t0 >> 1;
     const int side = (int)(t0 & 1);
     bool active = e0 < n_edge;
@@ -1122,11 +1152,12 @@ __global__ void __launch_bounds__(RT_THREADS, FR_EDGE_MIN_BLOCKS) k_edge_primary
     uint64_t vis[2];
     RayStats rs;
     __shared__ Cover cover[RT_WARPS];
-    const float3 L = radiance_at<ENV>(S, P, active, X + eps * mx, Y + eps * my, smp, 4, sh, cover[threadIdx.x >> 5],
-                                      my_stack(sh), ss, vis, rs);
+    const float3 L = radiance_at<ENV, SPLIT>(S, P, active, X + eps * mx, Y + eps * my, smp, 4, sh,
+                                             cover[threadIdx.x >> 5], my_stack(sh), ss, vis, rs);
     const float3 Lo = f3(__shfl_xor_sync(FULL, L.x, 1), __shfl_xor_sync(FULL, L.y, 1), __shfl_xor_sync(FULL, L.z, 1));
     const float3 Lp = side ? Lo : L, Lm = side ? L : Lo;
     if (side) active = false;                          // the even lane adds the pair's term
+    if (SPLIT > 1 && threadIdx.x >= 32) active = false;
     flush_stats(S.counters + 6, rs);
     float gf = 0.0f;
     float3 gA = f3(0, 0, 0), gB = f3(0, 0, 0);
@@ -1858,34 +1889,19 @@ int blocks_for(long n, int t) { return (int)((n + t - 1) / t); }
 // ---------------------------------------------------------------------------
 int map_blocks(const BlockMap& m) { return m.block0[m.n]; }
 
-// Shared-memory carveout of the ray kernels in percent (-1: the driver's
-// choice).  L1 holds the BVH nodes, triangles and local traversal stacks, so a
-// large carveout starves it.
-#ifndef FR_CARVEOUT
-#define FR_CARVEOUT -1
-#endif
-template <bool ENV>
-void set_carveout() {
-    static bool done = false;
-    if (done || FR_CARVEOUT < 0) return;
-    cudaFuncSetAttribute(k_forward<ENV>, cudaFuncAttributePreferredSharedMemoryCarveout, FR_CARVEOUT);
-    cudaFuncSetAttribute(k_adjoint<false, ENV>, cudaFuncAttributePreferredSharedMemoryCarveout, FR_CARVEOUT);
-    cudaFuncSetAttribute(k_adjoint<true, ENV>, cudaFuncAttributePreferredSharedMemoryCarveout, FR_CARVEOUT);
-    cudaFuncSetAttribute(k_edge_primary<ENV>, cudaFuncAttributePreferredSharedMemoryCarveout, FR_CARVEOUT);
-    done = true;
-}
-
 // env: some item of the launch has environment blocks (the kernels compiled
-// with their code); otherwise the light-stage-only instantiation runs.
-void launch_forward(const DevItem* items, const BlockMap& map, bool env, long q0, bool records_only,
+// with their code); otherwise the light-stage-only instantiation runs.  split:
+// the map gives each block 32 samples, whose shadow rays its warps share.
+void launch_forward(const DevItem* items, const BlockMap& map, bool env, bool split, long q0, bool records_only,
                     cudaStream_t st) {
-    if (map_blocks(map) == 0) return;
+    const int n = map_blocks(map), rec = records_only ? 1 : 0;
+    if (n == 0) return;
     if (env) {
-        set_carveout<true>();
-        k_forward<true><<<map_blocks(map), RT_THREADS, 0, st>>>(items, map, q0, records_only ? 1 : 0);
+        if (split) k_forward<true, RT_WARPS><<<n, RT_THREADS, 0, st>>>(items, map, q0, rec);
+        else k_forward<true, 1><<<n, RT_THREADS, 0, st>>>(items, map, q0, rec);
     } else {
-        set_carveout<false>();
-        k_forward<false><<<map_blocks(map), RT_THREADS, 0, st>>>(items, map, q0, records_only ? 1 : 0);
+        if (split) k_forward<false, RT_WARPS><<<n, RT_THREADS, 0, st>>>(items, map, q0, rec);
+        else k_forward<false, 1><<<n, RT_THREADS, 0, st>>>(items, map, q0, rec);
     }
     fr_count_launches(1);
 }
@@ -1914,12 +1930,17 @@ void launch_edge_order(const DevItem* items, int n, long max_edge, cudaStream_t 
     fr_count_launches(1);
 }
 
-void launch_edge_primary(const DevItem* items, const BlockMap& map, bool env, cudaStream_t st) {
-    if (map_blocks(map) == 0) return;
-    if (env)
-        k_edge_primary<true><<<map_blocks(map), RT_THREADS, sizeof(float) * RT_WARPS, st>>>(items, map);
-    else
-        k_edge_primary<false><<<map_blocks(map), RT_THREADS, sizeof(float) * RT_WARPS, st>>>(items, map);
+void launch_edge_primary(const DevItem* items, const BlockMap& map, bool env, bool split, cudaStream_t st) {
+    const int n = map_blocks(map);
+    if (n == 0) return;
+    const size_t acc = sizeof(float) * RT_WARPS;
+    if (env) {
+        if (split) k_edge_primary<true, RT_WARPS><<<n, RT_THREADS, acc, st>>>(items, map);
+        else k_edge_primary<true, 1><<<n, RT_THREADS, acc, st>>>(items, map);
+    } else {
+        if (split) k_edge_primary<false, RT_WARPS><<<n, RT_THREADS, acc, st>>>(items, map);
+        else k_edge_primary<false, 1><<<n, RT_THREADS, acc, st>>>(items, map);
+    }
     fr_count_launches(1);
 }
 
