@@ -261,9 +261,9 @@ fr_status fr_forward(fr_ctx* ctx, const fr_params* p, float* image, uint32_t ite
  * curve n_s . o = 0 of App. A, Eq. brdf_spec, met along one row line per
  * pixel row and one column line per pixel column, edge_spp of each, rows
  * first; (W + H) * max(edge_spp, 1) <= 65535) unless disabled by flags.
- * adj_image [H][W][3] (device).  The boundary terms of the primary edges and
- * of the specular cutoff, and the texture-gradient flush, run on a stream of
- * the context, forked from `stream` and joined back into it with events. */
+ * adj_image [H][W][3] (device).  The boundary term of the primary edges, the
+ * texture-gradient flush and the pose's sums run on a stream of the context,
+ * forked from `stream` and joined back into it with events. */
 fr_status fr_backward(fr_ctx* ctx, const fr_params* p, const float* adj_image, fr_grads* g,
                       uint32_t iteration, uint32_t face_id, void* stream);
 
@@ -283,10 +283,10 @@ fr_status fr_loss(fr_ctx* ctx, const float* image, const float* target, double* 
  * FR_FLAG_RECOMPUTE it re-traces every sample inside the adjoint kernel
  * instead.  The gradient is the same either
  * way.  With g, the part of the adjoint that needs only the posed geometry
- * runs on a stream of the context beside the forward, the boundary terms of
- * the primary edges and of the specular lobe's cutoff run there beside the
- * interior term, and the texture gradients are flushed there beside the chain
- * to the vertex parameters; each piece is forked from `stream` and joined back
+ * runs on a stream of the context beside the forward, the boundary term of
+ * the primary edges runs there beside the interior term, and the texture
+ * gradients are flushed and the pose's sums taken there beside the chain to the
+ * vertices and coefficients; each piece is forked from `stream` and joined back
  * into it with events before the call's last work on `stream` (the call still
  * returns without synchronising, and a stream capture of it records the forks
  * and joins). */
@@ -411,7 +411,7 @@ fr_status fr_set_timing(fr_ctx* ctx, int32_t on);
  * boundary terms (primary edges and the specular lobe's boundary), chain to
  * parameters, total}.  The marks are events on the caller's stream: work on
  * the context's side stream counts in the stage it overlaps (the
- * classification in the forward's, the boundary terms in the adjoint's), and
+ * classification in the forward's, the primary edges in the adjoint's), and
  * its own stage holds only what is left of it after that stage ends. */
 fr_status fr_get_timing(fr_ctx* ctx, float* out);
 

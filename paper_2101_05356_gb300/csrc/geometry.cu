@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(256) k_vertex_normals(const DevItem* items, co
 }
 
 // dE/dm_i = (I - n n^T) dE/dn_i / |m_i|
-__global__ void k_normals_adj_a(const DevItem* items, int N) {
+__global__ void k_normals_adj(const DevItem* items, int N) {
     const DevItem& it = items[blockIdx.y];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
@@ -152,36 +152,34 @@ __global__ void k_normals_adj_a(const DevItem* items, int N) {
     it.dm[3 * i] = r.x; it.dm[3 * i + 1] = r.y; it.dm[3 * i + 2] = r.z;
 }
 
-// Face normal n_f = (b - a) x (c - a) feeds m of its three vertices; gather the
-// cross-product adjoint back to each vertex over its faces.
-__global__ void k_normals_adj_b(const DevItem* items, const int4* __restrict__ faces, const int* __restrict__ off,
-                                const int* __restrict__ idx, int N) {
-    const DevItem& it = items[blockIdx.y];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const float* dm = it.dm;
-    const float4* v = it.v_cam;
-    float3 acc = f3(0.0f, 0.0f, 0.0f);
-    for (int k = off[i]; k < off[i + 1]; ++k) {
-        const int4 t = faces[idx[k]];
-        const float3 G = f3(dm[3 * t.x] + dm[3 * t.y] + dm[3 * t.z], dm[3 * t.x + 1] + dm[3 * t.y + 1] + dm[3 * t.z + 1],
-                            dm[3 * t.x + 2] + dm[3 * t.y + 2] + dm[3 * t.z + 2]);
-        const float3 a = xyz(v[t.x]), b = xyz(v[t.y]), c = xyz(v[t.z]);
-        const float3 gu = cross(c - a, G);     // d/d(b - a)
-        const float3 gw = cross(G, b - a);     // d/d(c - a)
-        if (i == t.x) acc -= gu + gw;
-        else if (i == t.y) acc += gu;
-        else acc += gw;
+// Sums of 16 values over the warp, value q left in lanes 2 q and 2 q + 1: the
+// lanes 16, 8, 4, 2 and 1 apart are added, the first four times handing half of
+// the values left to the other half of the lanes, so every sum is the
+// butterfly's bit for bit in 16 FP64 additions instead of 80.
+FR_D double warp_sums16(double (&v)[16]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int n = 8; n >= 1; n >>= 1, o >>= 1) {
+        const bool high = lane & o;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const double keep = high ? v[i + n] : v[i], send = high ? v[i] : v[i + n];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
     }
-    fix64* d_v = it.G.d_v;                       // one writer per vertex here
-    d_v[3 * i] += (fix64)to_fix(acc.x);
-    d_v[3 * i + 1] += (fix64)to_fix(acc.y);
-    d_v[3 * i + 2] += (fix64)to_fix(acc.z);
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-// dE/dv = R dE/dv'; per-block partials of M'[r][c] = sum_i g_r w_c and
-// sum_i g (FP64), summed in block order by k_pose_finish.
-__global__ void __launch_bounds__(256) k_pose_adj(const DevItem* items, int N) {
+// The vertex's gradient and its share of the pose's.  Face normal n_f = (b - a)
+// x (c - a) feeds m of its three vertices: the cross-product adjoint is gathered
+// back to the vertex over its faces and added to dE/dv' (the boundary and
+// interior terms' sum).  Then dE/dv = R dE/dv', and per-block partials of
+// M'[r][c] = sum_i g_r w_c and sum_i g (FP64), summed in block order by
+// k_pose_finish.  Bound by the latency of its gathers; one launch instead of two
+// keeps the vertex's gradient in registers (paper-scale face: 21 -> 12 us).
+__global__ void __launch_bounds__(256) k_vertex_adj(const DevItem* items, const int4* __restrict__ faces,
+                                                    const int* __restrict__ off, const int* __restrict__ idx, int N) {
     __shared__ float R[9], T[3];
     __shared__ double part[8][12];
     const DevItem& it = items[blockIdx.y];
@@ -189,25 +187,47 @@ __global__ void __launch_bounds__(256) k_pose_adj(const DevItem* items, int N) {
         euler_R(it.P.rot, R);
         T[0] = it.P.trans[0]; T[1] = it.P.trans[1]; T[2] = it.P.trans[2];
     }
-    __syncthreads();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    double loc[12];
-    for (int k = 0; k < 12; ++k) loc[k] = 0.0;
+    float3 acc = f3(0.0f, 0.0f, 0.0f);
+    if (i < N) {
+        const float* dm = it.dm;
+        const float4* v = it.v_cam;
+        for (int k = off[i]; k < off[i + 1]; ++k) {
+            const int4 t = faces[idx[k]];
+            const float3 G = f3(dm[3 * t.x] + dm[3 * t.y] + dm[3 * t.z], dm[3 * t.x + 1] + dm[3 * t.y + 1] + dm[3 * t.z + 1],
+                                dm[3 * t.x + 2] + dm[3 * t.y + 2] + dm[3 * t.z + 2]);
+            const float3 a = xyz(v[t.x]), b = xyz(v[t.y]), c = xyz(v[t.z]);
+            const float3 gu = cross(c - a, G);     // d/d(b - a)
+            const float3 gw = cross(G, b - a);     // d/d(c - a)
+            if (i == t.x) acc -= gu + gw;
+            else if (i == t.y) acc += gu;
+            else acc += gw;
+        }
+    }
+    __syncthreads();
+    double loc[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) loc[k] = 0.0;
     if (i < N) {
         const fix64* d_v = it.G.d_v;
         const float* vm = it.v_model;
-        const float g[3] = {(float)from_fix(d_v[3 * i]), (float)from_fix(d_v[3 * i + 1]), (float)from_fix(d_v[3 * i + 2])};
+        const float g[3] = {(float)from_fix(d_v[3 * i] + (fix64)to_fix(acc.x)),
+                            (float)from_fix(d_v[3 * i + 1] + (fix64)to_fix(acc.y)),
+                            (float)from_fix(d_v[3 * i + 2] + (fix64)to_fix(acc.z))};
         const float w[3] = {vm[3 * i] - T[0], vm[3 * i + 1] - T[1], vm[3 * i + 2] - T[2]};
+#pragma unroll
         for (int r = 0; r < 3; ++r)
+#pragma unroll
             for (int c = 0; c < 3; ++c) loc[3 * r + c] = (double)g[r] * (double)w[c];
+#pragma unroll
         for (int r = 0; r < 3; ++r) loc[9 + r] = g[r];
+#pragma unroll
         for (int c = 0; c < 3; ++c)
             it.d_vmodel[3 * i + c] = R[3 * c + 0] * g[0] + R[3 * c + 1] * g[1] + R[3 * c + 2] * g[2];
     }
-    for (int k = 0; k < 12; ++k)
-        for (int o = 16; o > 0; o >>= 1) loc[k] += __shfl_xor_sync(0xffffffffu, loc[k], o);
-    if ((threadIdx.x & 31) == 0)
-        for (int k = 0; k < 12; ++k) part[threadIdx.x >> 5][k] = loc[k];
+    const double sum = warp_sums16(loc);
+    const int lane = threadIdx.x & 31;
+    if ((lane & 1) == 0 && lane < 24) part[threadIdx.x >> 5][lane >> 1] = sum;
     __syncthreads();
     if (threadIdx.x < 12) {
         double s = 0.0;
@@ -372,16 +392,11 @@ void launch_vertex_normals(const DevItem* items, int n, const int* vf_off, const
     fr_count_launches(1);
 }
 
-void launch_normals_adjoint(const DevItem* items, int n, const int4* faces, const int* vf_off,
-                            const int* vf_idx, int N, cudaStream_t st) {
-    k_normals_adj_a<<<dim3(nb(N, 256), n), 256, 0, st>>>(items, N);
-    k_normals_adj_b<<<dim3(nb(N, 256), n), 256, 0, st>>>(items, faces, vf_off, vf_idx, N);
+void launch_vertex_adjoint(const DevItem* items, int n, const int4* faces, const int* vf_off, const int* vf_idx, int N,
+                           cudaStream_t st) {
+    k_normals_adj<<<dim3(nb(N, 256), n), 256, 0, st>>>(items, N);
+    k_vertex_adj<<<dim3(nb(N, 256), n), 256, 0, st>>>(items, faces, vf_off, vf_idx, N);
     fr_count_launches(2);
-}
-
-void launch_pose_adjoint(const DevItem* items, int n, int N, cudaStream_t st) {
-    k_pose_adj<<<dim3(nb(N, 256), n), 256, 0, st>>>(items, N);
-    fr_count_launches(1);
 }
 
 void launch_pose_finish(const DevItem* items, int n, int NL, int N, cudaStream_t st) {

@@ -18,9 +18,8 @@ void launch_stage_lights(const DevItem* items, int n, int NL, cudaStream_t st);
 void launch_faces(const DevItem* items, int n, const int4* faces, int T, cudaStream_t st);
 void launch_vertex_normals(const DevItem* items, int n, const int* vf_off, const int* vf_idx, int N,
                            cudaStream_t st);
-void launch_normals_adjoint(const DevItem* items, int n, const int4* faces, const int* vf_off,
-                            const int* vf_idx, int N, cudaStream_t st);
-void launch_pose_adjoint(const DevItem* items, int n, int N, cudaStream_t st);
+void launch_vertex_adjoint(const DevItem* items, int n, const int4* faces, const int* vf_off, const int* vf_idx, int N,
+                           cudaStream_t st);
 void launch_pose_finish(const DevItem* items, int n, int NL, int N, cudaStream_t st);
 
 // linear.cu: y_b = mean + basis * coef_b for the faces of a batch (shape morph,
