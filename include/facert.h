@@ -261,9 +261,10 @@ fr_status fr_forward(fr_ctx* ctx, const fr_params* p, float* image, uint32_t ite
  * curve n_s . o = 0 of App. A, Eq. brdf_spec, met along one row line per
  * pixel row and one column line per pixel column, edge_spp of each, rows
  * first; (W + H) * max(edge_spp, 1) <= 65535) unless disabled by flags.
- * adj_image [H][W][3] (device).  The boundary term of the primary edges, the
- * texture-gradient flush and the pose's sums run on a stream of the context,
- * forked from `stream` and joined back into it with events. */
+ * adj_image [H][W][3] (device).  The part that needs only the posed geometry,
+ * the boundary term of the primary edges, the texture-gradient flush and the
+ * pose's sums run on a stream of the context, forked from `stream` and joined
+ * back into it with events. */
 fr_status fr_backward(fr_ctx* ctx, const fr_params* p, const float* adj_image, fr_grads* g,
                       uint32_t iteration, uint32_t face_id, void* stream);
 

@@ -487,7 +487,21 @@ void adjoint_prep(fr_ctx* c, int n, cudaStream_t st) {
     launch_spec_candidates(c->d_items, n, c->T, spec_map(c, n), st);
 }
 
-// The rest of the reverse pass, after adjoint_prep and the loss.  The boundary
+// Fork adjoint_prep onto the context's side stream after the work already on
+// `st` (the built geometry); adjoint_main makes `st` wait for it (tail_ev).
+// Between the two the caller's stream runs the forward and the loss, or the
+// stand-alone adjoint's records-only pass, which share no buffer with
+// adjoint_prep.  Under stream capture the fork and join are part of the captured
+// graph.
+fr_status fork_prep(fr_ctx* c, int n, cudaStream_t st) {
+    CK(c, cudaEventRecord(c->fork_ev, st));
+    CK(c, cudaStreamWaitEvent(c->side, c->fork_ev, 0));
+    adjoint_prep(c, n, c->side);
+    CK(c, cudaEventRecord(c->tail_ev, c->side));
+    return FR_OK;
+}
+
+// The rest of the reverse pass, after fork_prep and the loss.  The boundary
 // terms (primary edges, the specular lobe's cutoff) and the interior term
 // (with the shadow-boundary term) only add into the fixed-point accumulators
 // with integer atomics, whose sums do not depend on their order, and read
@@ -518,6 +532,7 @@ fr_status adjoint_main(fr_ctx* c, int n, cudaStream_t st) {
     if (all_full || any_retrace) {
         // records of the whole image from this step's forward, or (some item
         // asked for it) re-tracing in the adjoint itself
+        CK(c, cudaStreamWaitEvent(st, c->tail_ev, 0));
         launch_adjoint(c->d_items, map_of(c, n, false), c->NL, all_full, any_stage, env, 0, st);
     } else {
         // recomputed records: per tile of `cap` camera samples, from the last
@@ -536,6 +551,7 @@ fr_status adjoint_main(fr_ctx* c, int n, cudaStream_t st) {
             const bool split = split_lights(c, n, map, split_forward(c));
             if (split) map = tile_map(c, n, q0, cap, lacks, 32);
             launch_forward(c->d_items, map, env, split, q0, true, st);
+            if (t == n_tiles - 1) CK(c, cudaStreamWaitEvent(st, c->tail_ev, 0));   // adjoint_prep
             launch_adjoint(c->d_items, tile_map(c, n, q0, cap, [](const DevItem&) { return true; }), c->NL, true,
                            any_stage, env, q0, st);
         }
@@ -560,30 +576,6 @@ fr_status adjoint_main(fr_ctx* c, int n, cudaStream_t st) {
     morph_adjoint(c, n, st);
     CK(c, cudaStreamWaitEvent(st, c->tail_ev, 0));
     mark(c, 7, st);
-    return FR_OK;
-}
-
-// reverse pass for items [0, n) whose geometry is built (adjoint_prep on `st`)
-fr_status adjoint_pass(fr_ctx* c, int n, cudaStream_t st) {
-    adjoint_prep(c, n, st);
-    return adjoint_main(c, n, st);
-}
-
-// Fork adjoint_prep onto the context's side stream after the work already on
-// `st` (the built geometry); join_prep makes `st` wait for it.  Between the two
-// the caller's stream runs the forward and the loss, which share no buffer
-// with adjoint_prep.  Under stream capture the fork and join are part of the
-// captured graph.
-fr_status fork_prep(fr_ctx* c, int n, cudaStream_t st) {
-    CK(c, cudaEventRecord(c->fork_ev, st));
-    CK(c, cudaStreamWaitEvent(c->side, c->fork_ev, 0));
-    adjoint_prep(c, n, c->side);
-    CK(c, cudaEventRecord(c->join_ev, c->side));
-    return FR_OK;
-}
-
-fr_status join_prep(fr_ctx* c, cudaStream_t st) {
-    CK(c, cudaStreamWaitEvent(st, c->join_ev, 0));
     return FR_OK;
 }
 
@@ -1047,7 +1039,8 @@ fr_status fr_backward(fr_ctx* c, const fr_params* p, const float* adj_image, fr_
     c->h_items[0] = make_item(c, 0, single(c, p, g, nullptr, adj_image, iteration, face_id));
     TRY(upload(c, 1, st));
     build_geometry(c, 1, st);
-    TRY(adjoint_pass(c, 1, st));
+    TRY(fork_prep(c, 1, st));
+    TRY(adjoint_main(c, 1, st));
     CK(c, cudaGetLastError());
     return FR_OK;
 }
@@ -1082,7 +1075,6 @@ fr_status fr_render(fr_ctx* c, const fr_params* p, const float* target, float* i
     launch_loss(loss_table(c, 1, tg, ls, g != nullptr), st);
     mark(c, 3, st);
     if (g) {
-        TRY(join_prep(c, st));
         TRY(adjoint_main(c, 1, st));
     }
     CK(c, cudaGetLastError());
@@ -1128,7 +1120,6 @@ fr_status fr_render_batch(fr_ctx* c, const fr_item* items, int32_t n, void* stre
             if (!items[k].grads)
                 CK(c, cudaMemsetAsync(c->slots[k].adj_image, 0,
                                       sizeof(float) * 3 * (size_t)items[k].width * items[k].height, st));
-        TRY(join_prep(c, st));
         TRY(adjoint_main(c, n, st));
     }
     CK(c, cudaGetLastError());
