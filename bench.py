@@ -48,7 +48,8 @@ METRIC = "rays/s fwd+adjoint"
 WORKLOAD = ("paper-scale single face: 35,709 verts / 70,789 tris, K=80+64, 256x256, 16 spp, "
             "40 quad lights, 512^2 textures, 1 primary-edge sample/pixel")
 # ALU work per traversal step (algorithmic op counts, FP32 lane operations):
-# a node visit tests two child boxes (2 x (6 FMA slab + 10 min/max/compare)),
+# a node visit tests two child boxes (2 x (6 FMA slab + 10 min/max/compare);
+# the shadow rays' two plane tests are not counted as work),
 # a Woop triangle test is ~30 operations (shear 6, edge functions 6, det 2,
 # distance 3, compares and the reciprocal ~13).
 OPS_PER_NODE = 32
@@ -57,13 +58,13 @@ OPS_PER_TRI = 30
 # kernel from one ncu capture of this benchmark's workload, valid while the
 # sources that make up the kernel hash to `sources_sha256` (else reported as
 # null); the capture command is recorded beside the kernel's profile summary.
-TRAFFIC = {"k_forward": {"bytes": 23236864 + 9601280,
-                         "sources_sha256": "292936dfbfa4dd07bcb5f6f205eda95c504a32d0849ea664c071a481b62b02fe"}}
+TRAFFIC = {"k_forward": {"bytes": 20503808 + 793600,
+                         "sources_sha256": "9f4469a1788b8b2e0d8e4da2a3e3d391ba980eb62e4789bc03e618d0c15ea1c1"}}
 KERNEL_SOURCES = {"k_forward": ("render.cu", "trace.cuh", "shade.cuh", "common.cuh")}
-# Issue-slot use (smsp__issue_active) of a kernel from its ncu --set full capture,
+# Issue-slot use (smsp__issue_active) of a kernel from the same capture,
 # valid while its sources hash to `sources_sha256`.
-ISSUE = {"k_forward": {"frac": 0.7020,
-                       "sources_sha256": "292936dfbfa4dd07bcb5f6f205eda95c504a32d0849ea664c071a481b62b02fe"}}
+ISSUE = {"k_forward": {"frac": 0.7037,
+                       "sources_sha256": "9f4469a1788b8b2e0d8e4da2a3e3d391ba980eb62e4789bc03e618d0c15ea1c1"}}
 FP32_LANES_PER_SM = 128
 
 

@@ -2,9 +2,9 @@
 // when the mesh is set (like the edge and vertex->face lists): a binned
 // surface-area-heuristic split of the mean face's triangles (model space),
 // single-triangle leaves, internal nodes numbered in pre-order (root 0) and
-// leaves numbered left to right.  Every call then refits the boxes of this
-// topology to the morphed, posed face on the GPU (k_boxes / k_pack in
-// lbvh.cu); the per-call LBVH rebuild remains available (FR_FLAG_LBVH) for
+// leaves numbered left to right.  Every call then refits the boxes and plane
+// bounds of this topology to the morphed, posed face on the GPU (k_pose_refit /
+// k_refit_top in refit.cu); the per-call LBVH rebuild remains available (FR_FLAG_LBVH) for
 // deformations the mean-face topology does not suit.
 //
 // Depth is capped: below depth SAH_MAX_DEPTH a node is split at the median of

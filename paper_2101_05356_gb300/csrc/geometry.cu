@@ -10,7 +10,7 @@
 
 namespace {
 
-// Items per k_set_items launch: 32 x 632-byte items stay under the 32 KB
+// Items per k_set_items launch: 32 x 760-byte items stay under the 32 KB
 // kernel-parameter limit.
 constexpr int ITEMS_PER_LAUNCH = 32;
 

@@ -1,10 +1,11 @@
 // Linear BVH over the camera-space triangles (the per-call rebuild; the
-// default refits a static SAH topology built at set-up, bvh_topology.cu, with
-// the same box and pack kernels): Morton keys
-// of the centroids (geometry.cu), a stable LSD radix sort (4 x 8-bit passes),
-// the radix-tree construction of Karras (HPG 2012) with index tie-breaks, and a
-// bottom-up box pass with one atomic flag per internal node.  Leaves are single
-// triangles; nodes store both children's boxes for two-wide tests.
+// default refits a static SAH topology built at set-up, bvh_topology.cu, in
+// refit.cu): Morton keys of the centroids (geometry.cu), a stable LSD radix sort
+// (4 x 8-bit passes), the radix-tree construction of Karras (HPG 2012) with
+// index tie-breaks, a bottom-up box pass with one atomic flag per internal node
+// and the plane bounds of the packed nodes (k_planes).  Leaves are single
+// triangles; nodes store both children's boxes and plane bounds for two-wide
+// tests.
 #include "common.cuh"
 #include "kernels.h"
 #include "refit.cuh"

@@ -29,8 +29,9 @@ constexpr int RT_WARPS = RT_THREADS / 32;
 // Measured on GB300 (paper-scale face): the forward is fastest at 8 blocks
 // (1.25 ms; 7: 1.30 ms, 9: 1.27 ms, 6: 1.37 ms), the primary-edge kernel at 7
 // (step 1.99 ms; 6 the same, at 512 x 512 4.44 ms against 4.46 ms), the
-// adjoint reading hit records at 5 (0.601 ms; 6: 0.618 ms, 8: 0.637 ms) and
-// the re-tracing adjoint at 8 (4.20 ms; 6: 4.38 ms, 5: 4.65 ms).
+// adjoint reading hit records at 5 (step 1.93 ms; 4 the same, 6: 1.95 ms, 8:
+// 1.98 ms) and the re-tracing adjoint at 8 (re-traced step 3.16 ms; 6: 3.165
+// ms, 5: 3.20 ms).
 #ifndef FR_FWD_MIN_BLOCKS
 #define FR_FWD_MIN_BLOCKS 8
 #endif
@@ -351,7 +352,6 @@ FR_D float3 radiance_from(const DevScene& S, const DevParams& P, const SampleSta
 
 // Warp-cooperative visibility at screen point (sx, sy): the camera ray's hit
 // (without the material) and both shadow-visibility words.
-FR_D void make_cover(const DevScene&, const SampleState&, NoCover&) {}
 FR_D void make_cover(const DevScene& S, const SampleState& ss, Cover& c) {
     build_cover(S, c, __ballot_sync(FULL, ss.hit && ss.lit), ss.slot);
 }

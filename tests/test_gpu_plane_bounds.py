@@ -1,10 +1,11 @@
 """The any-hit traversal culls a BVH node whose plane bound the ray stays above
-(csrc/refit.cu; csrc/lbvh.cu, k_planes).  A bound that cut off a triangle would lose shadows,
-so every sample's visibility words are compared with the oracle's brute force
-on triangle soups of the sizes where the bounds change hands: one and two
-triangles, the 8 a thread takes and one more, the 256 of a refit block and one
-more, the 4,096 a bound may span and more, at the face's scale and 50 times it, for both trees.  At most two
-samples may disagree (FP32 and FP64 flips at triangle edges).  Overlapping
+(csrc/refit.cu; csrc/lbvh.cu, k_planes).  A bound that cut off a triangle would
+lose shadows, so every sample's visibility words are compared with the oracle's
+brute force on triangle soups of the sizes where the bounds change hands: one
+and two triangles, the 8 a thread takes and one more, the 256 of a refit block
+and one more, the 4,096 a bound may span and more, at the face's scale and 50
+times it, for both trees.  At most two samples may disagree (FP32 and FP64 flips
+at triangle edges).  Overlapping
 triangles of one plane tie for the camera ray's closest hit, which FP32 and
 FP64 rounding then pick differently, so the flat soups compare the visibility
 where the two sides' hits are the same triangle."""
