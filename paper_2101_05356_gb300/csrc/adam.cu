@@ -12,6 +12,8 @@
 // the chromaticity term.  With one thread per element and the energies in FP64
 // that launch took 103 us there, nearly all of it FP64 instructions; measured
 // now 22 us, and 8 us the second (13.7 us with one element a thread).
+#include <cfloat>
+
 #include "../../include/facert.h"
 #include "common.cuh"
 #include "kernels.h"
@@ -145,7 +147,8 @@ FR_D void pair_add_product(Pair& s, float w, float x) {    // s += w x
     s.lo = __fadd_rn(s.lo, __fmaf_rn(w, x, -p));
 }
 
-// The energy of texel t in FP64, for texels whose FP32 products overflow.
+// The energy of texel t in FP64, for texels whose FP32 products, or the warp's
+// sum of them, would overflow.
 __device__ __noinline__ double texel_energy64(const fr_opt_group& G, int C, int t) {
     const int M = G.width;
     const int row = t / M, col = t - row * M;
@@ -295,7 +298,8 @@ __global__ void __launch_bounds__(ADAM_THREADS) k_adam_moments(GroupTable T, dou
         }
         if (ENERGY) {
             double wide = 0.0;
-            if (!isfinite(p.hi + p.lo)) {          // (an overflow of its products, or not a finite texel)
+            // (not a finite texel, an overflow of its products, or so large that the warp's 32 might overflow together)
+            if (!(fabsf(p.hi) < FLT_MAX / 64.0f)) {
                 wide = texel_energy64(G, G.kind == FR_GROUP_TEX_RGB ? 3 : 1, i);
                 p.hi = p.lo = 0.0f;
             }
