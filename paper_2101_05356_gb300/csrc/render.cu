@@ -1182,9 +1182,16 @@ __global__ void __launch_bounds__(RT_THREADS, FR_EDGE_MIN_BLOCKS) k_edge_primary
     }
     scatter_vertex(G.d_v, E.x, gA, active);
     scatter_vertex(G.d_v, E.y, gB, active);
+    // each warp's sum is rounded to fixed point by itself, so the total is the same
+    // whether a block holds four warps of samples or (SPLIT) one
     const float gw = warp_sum(gf);
     if ((threadIdx.x & 31) == 0) acc_dyn[threadIdx.x >> 5] = gw;
-    block_acc_flush(1, 0, 1, G.small);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        long long s = 0;
+        for (int w = 0; w < RT_WARPS; ++w) s += to_fix_d((double)acc_dyn[w]);
+        if (s != 0) atomicAdd(&G.small[0], (fix64)s);
+    }
 }
 
 // ---------------------------------------------------------------------------
