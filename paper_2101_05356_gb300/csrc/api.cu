@@ -7,6 +7,7 @@
 // is written to device memory by one small kernel, and every stage is one
 // launch over all items.  The single-face calls are batches of one.
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <atomic>
 #include <cstdio>
@@ -814,7 +815,20 @@ fr_status fr_set_mesh(fr_ctx* c, const fr_mesh* m) {
         CK(c, cudaMemcpy(d_treelets, treelets.data(), sizeof(Treelet) * treelets.size(), cudaMemcpyHostToDevice));
         if (!tops.empty())
             CK(c, cudaMemcpy(d_tops, tops.data(), sizeof(TopNode) * tops.size(), cudaMemcpyHostToDevice));
-        c->refit = RefitTopology{d_runs, d_treelets, d_tops, (int)treelets.size(), (int)tops.size()};
+        std::vector<float> reach(1 + (size_t)K, 0.0f);
+        for (int k = 0; k <= K; ++k) {
+            const float* col = k == 0 ? m->mean : m->basis + (size_t)(k - 1) * 3 * N;
+            for (int i = 0; i < N; ++i)
+                if (deg[i + 1] > deg[i]) {
+                    const float* x = col + 3 * (size_t)i;
+                    reach[k] = std::max(reach[k], x[0] * x[0] + x[1] * x[1] + x[2] * x[2]);
+                }
+            reach[k] = std::sqrt(reach[k]);
+        }
+        float* d_reach = nullptr;
+        TRY(dalloc(c, &d_reach, reach.size()));
+        CK(c, cudaMemcpy(d_reach, reach.data(), sizeof(float) * reach.size(), cudaMemcpyHostToDevice));
+        c->refit = RefitTopology{d_runs, d_treelets, d_tops, d_reach, (int)treelets.size(), (int)tops.size()};
     }
     TRY(dalloc(c, &c->faces, T));
     TRY(dalloc(c, &c->uv, N));

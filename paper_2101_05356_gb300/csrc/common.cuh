@@ -190,7 +190,7 @@ struct BvhScratch {
     float4* box_int;     // [2 (T - 1)] lo, hi; w: first leaf slot, leaf count (int bits)
     float4* box_leaf;    // [2 T]
     unsigned* aabb;      // [6] ordered-int scene bounds
-    float4* treelet_box; // [3 n_treelets] lo, hi, area vector of each treelet of the static topology
+    float4* treelet_box; // [3 n_treelets] lo, hi, area vector (w: the mesh's reach) of each treelet of the static topology
 };
 
 struct EdgeLists {

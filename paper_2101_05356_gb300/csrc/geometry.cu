@@ -53,14 +53,6 @@ __global__ void k_tex_flush(const DevItem* items, int M) {
     else if (it.G.roughness) it.G.roughness[i - 6 * M2] += g;
 }
 
-FR_D unsigned ordered(float f) {
-    const unsigned u = __float_as_uint(f);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-FR_D float unordered(unsigned u) {
-    return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
-}
-
 __global__ void k_aabb_reset(const DevItem* items) {
     unsigned* aabb = items[blockIdx.x].B.aabb;
     if (threadIdx.x < 3) aabb[threadIdx.x] = 0xffffffffu;

@@ -111,6 +111,7 @@ struct RefitTopology {
     const int2* runs;                    // [T - 1] each node's first leaf slot and leaf count
     const Treelet* treelets;
     const TopNode* tops;
+    const float* reach;                  // [1 + K] greatest length of the mean's and of each basis column's vectors, over the faces' vertices
     int n_treelets, n_tops;
 };
 void build_refit_lists(const BvhTopology& topo, int T, std::vector<int2>& runs, std::vector<Treelet>& treelets,

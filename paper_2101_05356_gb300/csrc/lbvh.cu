@@ -299,16 +299,16 @@ FR_D float3 area_vector(const float4* tris, int s) {
     return cross(xyz(tris[3 * s + 1]) - a, xyz(tris[3 * s + 2]) - a);
 }
 
-FR_D void plane_reach(const float4* tris, int s, float3 n, float& h, float& mag) {
+FR_D void plane_height(const float4* tris, int s, float3 n, float& h) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) plane_height(xyz(tris[3 * s + k]), n, h, mag);
+    for (int k = 0; k < 3; ++k) h = fmaxf(h, dot(n, xyz(tris[3 * s + k])));
 }
 
 // code >= 0: internal node, < 0: leaf ~slot; the child's record in its parent
-FR_D void store_plane(const BvhScratch& B, BvhNode* nodes, int code, float3 n, float h, float mag) {
+FR_D void store_plane(const BvhScratch& B, BvhNode* nodes, int code, float3 n, float h, float reach) {
     const int p = code < 0 ? B.parent_leaf[~code] : B.parent_int[code];
     if (p < 0) return;                                  // an invalid tree (its status is set): no record
-    const float4 v = plane_record(n, h, mag);
+    const float4 v = plane_record(n, h, reach);
     (B.child[2 * p] == code ? nodes[p].p0 : nodes[p].p1) = v;
 }
 
@@ -318,11 +318,13 @@ __global__ void __launch_bounds__(256) k_planes(const DevItem* items, int n) {
     const float4* __restrict__ tris = it.tris;
     const int lane = threadIdx.x & 31, n_warps = gridDim.x * (blockDim.x >> 5);
     const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    float reach = 0.0f;                                 // greatest coordinate of the posed mesh
+    for (int k = 0; k < 6; ++k) reach = fmaxf(reach, fabsf(unordered(B.aabb[k])));
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {    // leaves
         const float3 m = unit_or_zero(area_vector(tris, s));
-        float h = -INFINITY, mag = 0.0f;
-        plane_reach(tris, s, m, h, mag);
-        store_plane(B, it.nodes, ~s, m, h, mag);
+        float h = -INFINITY;
+        plane_height(tris, s, m, h);
+        store_plane(B, it.nodes, ~s, m, h, reach);
     }
     for (int i0 = w; i0 < n - 1; i0 += 32 * n_warps) {                                           // warp-uniform
         const int i = i0 + lane * n_warps;
@@ -337,9 +339,9 @@ __global__ void __launch_bounds__(256) k_planes(const DevItem* items, int n) {
             float3 m = f3(0.0f, 0.0f, 0.0f);
             for (int s = first; s < first + count; ++s) m += area_vector(tris, s);
             m = unit_or_zero(m);
-            float h = -INFINITY, mag = 0.0f;
-            for (int s = first; s < first + count; ++s) plane_reach(tris, s, m, h, mag);
-            store_plane(B, it.nodes, i, m, h, mag);
+            float h = -INFINITY;
+            for (int s = first; s < first + count; ++s) plane_height(tris, s, m, h);
+            store_plane(B, it.nodes, i, m, h, reach);
         }
         unsigned big = __ballot_sync(0xffffffffu, count > PLANE_THREAD && count <= PLANE_MAX);
         while (big) {
@@ -355,14 +357,11 @@ __global__ void __launch_bounds__(256) k_planes(const DevItem* items, int n) {
                 m.z += __shfl_xor_sync(0xffffffffu, m.z, o);
             }
             m = unit_or_zero(m);
-            float h = -INFINITY, mag = 0.0f;
-            for (int s = f + lane; s < f + c; s += 32) plane_reach(tris, s, m, h, mag);
+            float h = -INFINITY;
+            for (int s = f + lane; s < f + c; s += 32) plane_height(tris, s, m, h);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                h = fmaxf(h, __shfl_xor_sync(0xffffffffu, h, o));
-                mag = fmaxf(mag, __shfl_xor_sync(0xffffffffu, mag, o));
-            }
-            if (lane == src) store_plane(B, it.nodes, i, m, h, mag);
+            for (int o = 16; o > 0; o >>= 1) h = fmaxf(h, __shfl_xor_sync(0xffffffffu, h, o));
+            if (lane == src) store_plane(B, it.nodes, i, m, h, reach);
         }
     }
 }

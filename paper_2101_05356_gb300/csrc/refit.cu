@@ -59,10 +59,8 @@ struct Reach {
     }
 };
 
-FR_D void height_of(const Tri3& t, float3 n, float& h, float& mag) {
-    plane_height(t.a, n, h, mag);
-    plane_height(t.b, n, h, mag);
-    plane_height(t.c, n, h, mag);
+FR_D void height_of(const Tri3& t, float3 n, float& h) {
+    h = fmaxf(h, fmaxf(dot(n, t.a), fmaxf(dot(n, t.b), dot(n, t.c))));
 }
 
 FR_D float warp_min(float v) {
@@ -142,7 +140,7 @@ FR_D void vertex_and_normal(const DevItem& it, const float* R, const float* T, c
     it.vn[i] = vertex_normal(m);
 }
 
-FR_D void refit_treelet(const DevItem& it, TreeletShared& sh, const float* R, const float* T,
+FR_D void refit_treelet(const DevItem& it, TreeletShared& sh, const float* R, const float* T, float reach,
                         const int4* __restrict__ faces, const RefitTopology& topo, int k) {
     const Treelet tl = topo.treelets[k];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -159,9 +157,9 @@ FR_D void refit_treelet(const DevItem& it, TreeletShared& sh, const float* R, co
 #pragma unroll
         for (int c = 0; c < 9; ++c) sh.v[c][t] = w[c];
         const float3 n = unit_or_zero(cross(q.b - q.a, q.c - q.a));
-        float h = -INFINITY, mag = 0.0f;
-        height_of(q, n, h, mag);
-        const float4 p = plane_record(n, h, mag);
+        float h = -INFINITY;
+        height_of(q, n, h);
+        const float4 p = plane_record(n, h, reach);
         sh.leaf_plane[0][t] = p.x; sh.leaf_plane[1][t] = p.y; sh.leaf_plane[2][t] = p.z; sh.leaf_plane[3][t] = p.w;
     }
     __syncthreads();
@@ -177,9 +175,9 @@ FR_D void refit_treelet(const DevItem& it, TreeletShared& sh, const float* R, co
             r.clear();
             for (int l = run.x; l < run.x + run.y; ++l) r.add(shared_tri(sh, l));
             const float3 n = unit_or_zero(r.m);
-            float h = -INFINITY, mag = 0.0f;
-            for (int l = run.x; l < run.x + run.y; ++l) height_of(shared_tri(sh, l), n, h, mag);
-            put_node(sh, j, r.box, plane_record(n, h, mag));
+            float h = -INFINITY;
+            for (int l = run.x; l < run.x + run.y; ++l) height_of(shared_tri(sh, l), n, h);
+            put_node(sh, j, r.box, plane_record(n, h, reach));
         }
         unsigned big = __ballot_sync(0xffffffffu, run.y > NODE_THREAD);
         while (big) {
@@ -191,14 +189,13 @@ FR_D void refit_treelet(const DevItem& it, TreeletShared& sh, const float* R, co
             for (int l = f + lane; l < f + c; l += 32) r.add(shared_tri(sh, l));
             warp_reach(r);
             const float3 n = unit_or_zero(r.m);
-            float h = -INFINITY, mag = 0.0f;
-            for (int l = f + lane; l < f + c; l += 32) height_of(shared_tri(sh, l), n, h, mag);
+            float h = -INFINITY;
+            for (int l = f + lane; l < f + c; l += 32) height_of(shared_tri(sh, l), n, h);
             h = warp_max(h);
-            mag = warp_max(mag);
             if (lane == src) {
-                put_node(sh, j, r.box, plane_record(n, h, mag));
+                put_node(sh, j, r.box, plane_record(n, h, reach));
                 if (j == 0) {                     // the treelet's area vector, for the nodes above
-                    it.B.treelet_box[3 * k + 2] = make_float4(r.m.x, r.m.y, r.m.z, 0.0f);
+                    it.B.treelet_box[3 * k + 2] = make_float4(r.m.x, r.m.y, r.m.z, reach);
                 }
             }
         }
@@ -208,7 +205,7 @@ FR_D void refit_treelet(const DevItem& it, TreeletShared& sh, const float* R, co
                 const Tri3 q = shared_tri(sh, l);
                 m += cross(q.b - q.a, q.c - q.a);
             }
-            it.B.treelet_box[3 * k + 2] = make_float4(m.x, m.y, m.z, 0.0f);
+            it.B.treelet_box[3 * k + 2] = make_float4(m.x, m.y, m.z, reach);
         }
     }
     __syncthreads();
@@ -246,19 +243,34 @@ FR_D void refit_treelet(const DevItem& it, TreeletShared& sh, const float* R, co
     }
 }
 
+// Bounds the distance of every vertex of the posed mesh from the camera (a whole
+// warp calls): the mean's greatest length plus each basis column's times its
+// coefficient (1%: the sums' rounding and the BF16 morph's), moved by the
+// translation.
+FR_D float mesh_reach(const DevItem& it, const float* __restrict__ reach) {
+    const int lane = threadIdx.x & 31;
+    float r = lane == 0 ? reach[0] : 0.0f;
+    for (int k = lane; k < it.S.K; k += 32) r += fabsf(it.P.coef[k]) * reach[1 + k];
+    const float* t = it.P.trans;
+    return 1.01f * (warp_add(r) + sqrtf(t[0] * t[0] + t[1] * t[1] + t[2] * t[2]));
+}
+
 __global__ void __launch_bounds__(REFIT_THREADS) k_pose_refit(const DevItem* items, const int4* __restrict__ faces,
                                                               const int* __restrict__ off, const int* __restrict__ idx,
                                                               RefitTopology topo, int N) {
     __shared__ TreeletShared sh;
-    __shared__ float R[9], T[3];
+    __shared__ float R[9], T[3], reach;
     const DevItem& it = items[blockIdx.y];
     if (threadIdx.x == 0) {
         euler_R(it.P.rot, R);
         T[0] = it.P.trans[0]; T[1] = it.P.trans[1]; T[2] = it.P.trans[2];
+    } else if (threadIdx.x >> 5 == 1 && (int)blockIdx.x < topo.n_treelets) {
+        const float r = mesh_reach(it, topo.reach);
+        if ((threadIdx.x & 31) == 0) reach = r;
     }
     __syncthreads();
     if ((int)blockIdx.x < topo.n_treelets) {
-        refit_treelet(it, sh, R, T, faces, topo, blockIdx.x);
+        refit_treelet(it, sh, R, T, reach, faces, topo, blockIdx.x);
     } else {
         const int i = ((int)blockIdx.x - topo.n_treelets) * REFIT_THREADS + threadIdx.x;
         if (i < N) vertex_and_normal(it, R, T, faces, off, idx, i);
@@ -297,26 +309,20 @@ __global__ void __launch_bounds__(TOP_THREADS) k_refit_top(const DevItem* items,
     }
     const bool bound = u.count <= PLANE_MAX;       // block-uniform
     const float3 n = bound ? unit_or_zero(r.m) : f3(0.0f, 0.0f, 0.0f);
-    float h = -INFINITY, mag = 0.0f;
+    float h = -INFINITY;
     if (bound) {
         for (int s = u.first + t; s < u.first + u.count; s += TOP_THREADS)
-            height_of({xyz(it.tris[3 * s]), xyz(it.tris[3 * s + 1]), xyz(it.tris[3 * s + 2])}, n, h, mag);
+            height_of({xyz(it.tris[3 * s]), xyz(it.tris[3 * s + 1]), xyz(it.tris[3 * s + 2])}, n, h);
         h = warp_max(h);
-        mag = warp_max(mag);
         __syncthreads();                           // red is read above
-        if (lane == 0) {
-            red[warp][0] = h;
-            red[warp][1] = mag;
-        }
+        if (lane == 0) red[warp][0] = h;
         __syncthreads();
     }
     if (t == 0) {
         if (bound)
-            for (int w = 0; w < TOP_THREADS / 32; ++w) {
-                h = fmaxf(h, red[w][0]);
-                mag = fmaxf(mag, red[w][1]);
-            }
-        store_child(it.nodes[u.up >> 1], u.up & 1, r.box, plane_record(n, h, mag));
+            for (int w = 0; w < TOP_THREADS / 32; ++w) h = fmaxf(h, red[w][0]);
+        const float reach = it.B.treelet_box[3 * u.treelet + 2].w;
+        store_child(it.nodes[u.up >> 1], u.up & 1, r.box, plane_record(n, h, reach));
     }
 }
 

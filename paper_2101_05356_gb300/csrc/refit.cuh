@@ -8,6 +8,14 @@
 // the forward is 0.04 ms slower, with 65,536 as long as with 4,096.
 constexpr int PLANE_MAX = 4096;
 
+FR_D unsigned ordered(float f) {
+    const unsigned u = __float_as_uint(f);
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+FR_D float unordered(unsigned u) {
+    return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
+}
+
 // R = Rz(t2) Ry(t1) Rx(t0), row-major
 FR_D void euler_R(const float* rot, float R[9]) {
     float sx, cx, sy, cy, sz, cz;
@@ -78,16 +86,12 @@ FR_D float3 unit_or_zero(float3 m) {
     return l > 0.0f && l < INFINITY ? m * (1.0f / l) : f3(0.0f, 0.0f, 0.0f);
 }
 
-FR_D void plane_height(float3 p, float3 n, float& h, float& mag) {
-    h = fmaxf(h, dot(n, p));
-    mag = fmaxf(mag, fmaxf(fabsf(p.x), fmaxf(fabsf(p.y), fabsf(p.z))));
-}
-
-// The plane bound of a node with unit mean normal n (zero: none), greatest
-// height h = max n . x and greatest coordinate magnitude mag over its vertices.
-// The pad covers the rounding of both sides of the test (a few 2^-24 of the
-// coordinates' magnitude), as the boxes' does.
-FR_D float4 plane_record(float3 n, float h, float mag) {
+// The plane bound of a node with unit mean normal n (zero: none) and greatest
+// height h = max n . x over its vertices.  The pad covers the rounding of both
+// sides of the test, a few 2^-24 of the coordinates' magnitude: not of the
+// node's only, since a shadow ray's height is rounded at its origin's, which may
+// lie far beyond the node, so `reach` bounds the whole mesh's.
+FR_D float4 plane_record(float3 n, float h, float reach) {
     const bool none = n.x == 0.0f && n.y == 0.0f && n.z == 0.0f;
-    return make_float4(n.x, n.y, n.z, none ? 1.0f : h + 1e-5f + 1e-6f * mag);
+    return make_float4(n.x, n.y, n.z, none ? 1.0f : h + 1e-5f + 1e-6f * reach);
 }

@@ -100,9 +100,10 @@ FR_D bool box_hit(const RayPre& r, float3 lo, float3 hi, float tmin, float tmax,
 
 // Does the ray run above the plane bound (n, h) of a node all along [tn, tf],
 // the part of it inside the node's box?  The ends of that part are exact enough
-// for any hit on the node's triangles to lie between them (the box is padded by
-// more than their rounding), and the ray's height over the plane is linear.
-// A NaN height culls nothing.
+// for any hit on the node's triangles to lie between them (the bound is padded by
+// more than their rounding and the height's, plane_record), and the ray's height
+// over the plane is linear.  A height that is NaN at both ends culls nothing; at
+// one end only it is 0 * infinity, b = 0, and the other end's holds all along.
 FR_D bool above_plane(const RayPre& r, float4 p, float tn, float tf) {
     const float a = fmaf(p.x, r.o.x, fmaf(p.y, r.o.y, p.z * r.o.z));
     const float b = fmaf(p.x, r.d.x, fmaf(p.y, r.d.y, p.z * r.d.z));
