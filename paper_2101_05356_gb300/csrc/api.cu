@@ -483,7 +483,7 @@ void adjoint_prep(fr_ctx* c, int n, cudaStream_t st) {
         need_edges |= !(s.flags & FR_FLAG_NO_PRIMARY_EDGE) || !(s.flags & FR_FLAG_NO_SHADOW_EDGE);
         if (!(s.flags & FR_FLAG_NO_PRIMARY_EDGE)) max_edge = std::max(max_edge, (long)s.W * s.H * s.edge_spp);
     }
-    if (need_edges) launch_classify(c->d_items, n, c->E, c->NL, c->T, st);
+    if (need_edges) launch_classify(c->d_items, n, c->E, c->NL, c->T, c->env_size > 0, st);
     launch_edge_order(c->d_items, n, max_edge, st);
     launch_spec_candidates(c->d_items, n, c->T, spec_map(c, n), st);
 }
@@ -1251,7 +1251,7 @@ fr_status fr_debug_silhouettes(fr_ctx* c, const fr_params* p, int32_t* prim, int
     c->h_items[0] = make_item(c, 0, single(c, p, nullptr, nullptr, nullptr, 0, 0));
     TRY(upload(c, 1, st));
     build_geometry(c, 1, st);
-    launch_classify(c->d_items, 1, c->E, c->NL, c->T, st);
+    launch_classify(c->d_items, 1, c->E, c->NL, c->T, c->env_size > 0, st);
     const Slot& sl = c->slots[0];
     if (prim) CK(c, cudaMemcpyAsync(prim, sl.lists, sizeof(int) * c->E, cudaMemcpyDeviceToDevice, st));
     if (n_prim) CK(c, cudaMemcpyAsync(n_prim, sl.counts, sizeof(int), cudaMemcpyDeviceToDevice, st));
