@@ -322,18 +322,32 @@ BlockMap map_of(const fr_ctx* c, int n, bool edges, int per = 128) {
 // Few blocks: their warps then share the shadow rays of 32 samples instead of
 // holding 32 samples each, so that four times the warps cover the latency of
 // the walks, and the longest chain of walks is a quarter as long (they trace the
-// camera rays four times).  The lines, in blocks per SM of the unsplit launch,
-// lie where both sides were measured equal: forward at 8 lights 128 blocks 0.141
-// -> 0.098 ms, 512 blocks 0.137 -> 0.113, 800 blocks 0.143 -> 0.133, 1,280 blocks
-// 0.172 -> 0.193; at 40 lights 1,024 blocks 0.541 -> 0.406, 1,600 blocks 0.61 ->
-// 0.53, 1,967 blocks 0.65 -> 0.71; 64 environment blocks, 1,024 blocks, forward
-// and its records-only pass 2.88 -> 2.13 ms.  Primary edges
-// (the step's time): 64 blocks at 40 lights 0.87 -> 0.53 ms with the forward's,
-// 256 blocks at 40 lights 0.97 -> 0.85, 640 blocks at 8 lights 0.49 -> 0.52,
-// 1,024 blocks at 40 lights 1.99 -> 2.08.
-constexpr int SPLIT_FORWARD = 8, SPLIT_FORWARD_MANY = 11, SPLIT_MANY_LIGHTS = 32, SPLIT_EDGE = 4;
+// camera rays four times, and a warp takes two lights at least: one or two lights
+// leave the others idle).  The lines, in blocks per SM of the unsplit launch by
+// light count, lie where both sides were measured equal (split / unsplit, small
+// and paper-scale face, four poses).  Forward: 1 light 1.09 and 1.06 at 2 blocks
+// per SM, 1.47 and 1.35 at 8; 2 lights 0.97 and 1.02 at 1; 4 lights 1.03 and 1.01
+// at 4, 1.13 and 1.06 at 5; 6 lights 1.02 and 0.96 at 5, 8 lights 0.98 and 1.01,
+// 1.08 and 1.11 at 7; 12 lights 1.02 and 0.94 at 7; 16 lights 1.07 and 0.88 at 8;
+// 24 lights 1.01 and 0.99 at 10; 32 lights 0.93 and 0.91 at 11; 40 lights 0.98 and
+// 0.93 at 12, 1.06 and 1.00 at 14; 64 lights 0.97 and 0.91 at 14, but 64
+// environment blocks 0.97 and 0.85 at 11, 1.12 and 1.06 at 14.  Primary edges
+// (the step's time): up to 3 lights 1.00 at 1 and 1.14 and 1.09 at 4; 4 lights 0.99
+// at 1, 8 lights 0.97 and 0.97, 1.03 and 1.00 at 2; 12 lights 1.01 and 0.98 at 2,
+// 24 lights 0.97 and 0.96; 32 lights 1.02 and 0.97 at 3; 64 lights 1.02 and 0.98
+// at 4.
+struct SplitLine {
+    int lights, forward, edges;          // from this many lights on: blocks per SM of either launch
+};
+constexpr SplitLine SPLIT_LINES[] = {{0, 0, 0}, {2, 1, 0}, {4, 4, 1}, {6, 5, 1}, {12, 7, 2}, {16, 8, 2},
+                                     {24, 10, 2}, {32, 11, 3}, {40, 12, 3}, {64, 12, 4}};
 
-int split_forward(const fr_ctx* c) { return c->NL >= SPLIT_MANY_LIGHTS ? SPLIT_FORWARD_MANY : SPLIT_FORWARD; }
+SplitLine split_line(const fr_ctx* c) {
+    SplitLine line = SPLIT_LINES[0];
+    for (const SplitLine& l : SPLIT_LINES)
+        if (c->NL >= l.lights) line = l;
+    return line;
+}
 
 bool split_lights(const fr_ctx* c, int n, const BlockMap& unsplit, int per_sm) {
     for (int k = 0; k < n; ++k)
@@ -464,7 +478,7 @@ fr_status forward_pass(fr_ctx* c, int n, cudaStream_t st) {
         if (it.S.spp > 128) CK(c, cudaMemsetAsync(it.image, 0, sizeof(float) * 3 * (size_t)it.S.W * it.S.H, st));
     }
     BlockMap map = map_of(c, n, false);
-    const bool split = split_lights(c, n, map, split_forward(c));
+    const bool split = split_lights(c, n, map, split_line(c).forward);
     if (split) map = map_of(c, n, false, 32);
     launch_forward(c->d_items, map, c->env_size > 0, split, 0, false, st);
     return FR_OK;
@@ -516,7 +530,7 @@ fr_status adjoint_main(fr_ctx* c, int n, cudaStream_t st) {
     CK(c, cudaEventRecord(c->fork_ev, st));
     CK(c, cudaStreamWaitEvent(c->side, c->fork_ev, 0));
     BlockMap emap = map_of(c, n, true);
-    const bool esplit = split_lights(c, n, emap, SPLIT_EDGE);
+    const bool esplit = split_lights(c, n, emap, split_line(c).edges);
     if (esplit) emap = map_of(c, n, true, 32);
     launch_edge_primary(c->d_items, emap, c->env_size > 0, esplit, c->side);
     CK(c, cudaEventRecord(c->join_ev, c->side));
@@ -549,7 +563,7 @@ fr_status adjoint_main(fr_ctx* c, int n, cudaStream_t st) {
             const long q0 = t * cap;
             const auto lacks = [q0](const DevItem& it) { return !it.rec_full && it.rec_from != q0; };
             BlockMap map = tile_map(c, n, q0, cap, lacks);
-            const bool split = split_lights(c, n, map, split_forward(c));
+            const bool split = split_lights(c, n, map, split_line(c).forward);
             if (split) map = tile_map(c, n, q0, cap, lacks, 32);
             launch_forward(c->d_items, map, env, split, q0, true, st);
             if (t == n_tiles - 1) CK(c, cudaStreamWaitEvent(st, c->tail_ev, 0));   // adjoint_prep
