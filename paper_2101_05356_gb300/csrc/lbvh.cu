@@ -6,6 +6,8 @@
 // and the plane bounds of the packed nodes (k_planes).  Leaves are single
 // triangles; nodes store both children's boxes and plane bounds for two-wide
 // tests.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "refit.cuh"
@@ -282,16 +284,21 @@ __global__ void __launch_bounds__(256) k_pack(const DevItem* items, int n) {
 // shadow ray skims such patches all along its way over the face; over a plane
 // bound it passes clear of the whole patch (measured on the paper-scale face:
 // 17.7 node visits and 0.2 triangle tests per shadow ray against 36.1 and 4.4).
-// A node of more than PLANE_MAX triangles is too curved for a bound to cull and
-// keeps none (n = 0, h = 1): with a limit of 1,024 the forward is 0.04 ms slower
-// there, with 65,536 this kernel takes 0.4 ms more and the forward as long.
+// A node of more than `limit` triangles keeps none (n = 0, h = 1).
 //
-// Bound by the latency of its loads (every level of the tree reads all the
-// triangles once, from L2): about 0.03 ms on 70,789 triangles.  One thread takes
-// a node of up to PLANE_THREAD triangles (2 and 16 measure the same), the warp
-// together a larger one (its leaf slots are consecutive, so lanes read
-// neighbouring triangles).  Lane l of warp w owns node w + l * (number of warps):
-// the large nodes of the pre-order numbering's first chain land in different warps.
+// Bound by the latency of a warp's chain of nodes (every level of the tree reads
+// all the triangles once, from L2).  One thread takes a node of up to PLANE_THREAD
+// triangles (2 and 4 measure the same), the warp together a larger one (its leaf
+// slots are consecutive, so lanes read neighbouring triangles).  Lane l of warp w
+// owns node w + l * (number of warps): the large nodes of the pre-order
+// numbering's first chain land in different warps, and the launch has up to a
+// warp per node, as many as 1,024 blocks, so that few nodes follow each other in
+// one.  The build without this kernel: 0.146 ms on 5,120 triangles, 0.183 on
+// 70,789; with 32 nodes a warp and bounds over up to 4,096 triangles 0.191 and
+// 0.248, over 512 0.168 and 0.210; spread 0.155 over 512, 0.211 over 1,024.  The
+// limit, by the forward: 5,120 triangles, 8 lights, 16 samples a pixel of 256 x 256
+// 0.526 ms with 512, 0.531 with 1,024; 70,789 triangles, 40 lights 1.72 with 512,
+// 1.70 with 1,024 and 1.71 with 4,096 (a large tree's nodes are flatter).
 constexpr int PLANE_THREAD = 8;
 
 FR_D float3 area_vector(const float4* tris, int s) {
@@ -312,7 +319,7 @@ FR_D void store_plane(const BvhScratch& B, BvhNode* nodes, int code, float3 n, f
     (B.child[2 * p] == code ? nodes[p].p0 : nodes[p].p1) = v;
 }
 
-__global__ void __launch_bounds__(256) k_planes(const DevItem* items, int n) {
+__global__ void __launch_bounds__(256) k_planes(const DevItem* items, int n, int limit) {
     const DevItem& it = items[blockIdx.y];
     const BvhScratch& B = it.B;
     const float4* __restrict__ tris = it.tris;
@@ -333,7 +340,7 @@ __global__ void __launch_bounds__(256) k_planes(const DevItem* items, int n) {
             first = __float_as_int(B.box_int[2 * i].w);
             count = __float_as_int(B.box_int[2 * i + 1].w);
             if (first < 0 || count < 0 || count > n - first) count = 0;     // an invalid tree
-            if (count > PLANE_MAX) store_plane(B, it.nodes, i, f3(0.0f, 0.0f, 0.0f), 0.0f, 0.0f);
+            if (count > limit) store_plane(B, it.nodes, i, f3(0.0f, 0.0f, 0.0f), 0.0f, 0.0f);
         }
         if (count > 0 && count <= PLANE_THREAD) {
             float3 m = f3(0.0f, 0.0f, 0.0f);
@@ -343,7 +350,7 @@ __global__ void __launch_bounds__(256) k_planes(const DevItem* items, int n) {
             for (int s = first; s < first + count; ++s) plane_height(tris, s, m, h);
             store_plane(B, it.nodes, i, m, h, reach);
         }
-        unsigned big = __ballot_sync(0xffffffffu, count > PLANE_THREAD && count <= PLANE_MAX);
+        unsigned big = __ballot_sync(0xffffffffu, count > PLANE_THREAD && count <= limit);
         while (big) {
             const int src = __ffs(big) - 1;
             big &= big - 1;
@@ -368,8 +375,8 @@ __global__ void __launch_bounds__(256) k_planes(const DevItem* items, int n) {
 
 void launch_planes(const DevItem* items, int n, int T, cudaStream_t st) {
     if (T < 2) return;
-    // two nodes (an internal one and a leaf) a thread
-    k_planes<<<dim3((T + 255) / 256, n), 256, 0, st>>>(items, T);
+    const int blocks = std::max((T + 255) / 256, std::min(std::max(1024 / n, 1), (T + 7) / 8));
+    k_planes<<<dim3(blocks, n), 256, 0, st>>>(items, T, T < 16384 ? 512 : 1024);
     fr_count_launches(1);
 }
 

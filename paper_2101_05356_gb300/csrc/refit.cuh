@@ -3,11 +3,6 @@
 #pragma once
 #include "common.cuh"
 
-// A node of more triangles than this is too curved for a plane bound to cull
-// and keeps none (n = 0, h = 1).  Measured on the paper-scale face: with 1,024
-// the forward is 0.04 ms slower, with 65,536 as long as with 4,096.
-constexpr int PLANE_MAX = 4096;
-
 FR_D unsigned ordered(float f) {
     const unsigned u = __float_as_uint(f);
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
