@@ -40,3 +40,29 @@ def test_focal_gradient_alone_and_in_a_batch(n_lights):
             assert float(grads["focal"].abs()) > 0.0
             assert torch.equal(it["grads"]["focal"], grads["focal"]), (it["grads"]["focal"], grads["focal"])
     assert r.status() == 0
+
+
+@pytest.mark.parametrize("spp", [1, 2, 4, 32])
+@pytest.mark.parametrize("n_lights", [2, 5, 11, 40, 66])
+def test_image_alone_and_in_a_batch(n_lights, spp):
+    """One sample a pixel (32 pixels a block of the split form) to 32, with light counts from every part of the lines."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2101_05356_gb300 import facert
+    n = 64
+    w, h = {1: (83, 75), 2: (61, 56), 4: (45, 41), 32: (17, 15)}[spp]
+    sc = synth.make_scene("tiny", width=w, height=h, spp=spp, n_lights=n_lights)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    blocks = (w * h * spp + 127) // 128
+    assert blocks <= sms and n * blocks > 16 * sms
+    r = facert.Renderer(sc, max_batch=n)
+    p = r.device_params(synth.random_params(sc, 2))
+    tgt = torch.zeros(h, w, 3, device="cuda")
+    image, _, _ = r.render(p, tgt, iteration=3, with_grad=False)
+    items = [dict(width=w, height=h, spp=spp, edge_spp=1, iteration=3, face_id=0, params=p, target=tgt,
+                  image=torch.full((h, w, 3), -1.0, device="cuda"), loss=torch.zeros(1, dtype=torch.float64, device="cuda"),
+                  grads=None) for _ in range(n)]
+    facert.fr_render_batch(r.ctx, items)
+    for it in (items[0], items[n // 2], items[-1]):
+        assert torch.equal(it["image"], image)
+    assert float(image.abs().sum()) > 0.0 and r.status() == 0
