@@ -325,8 +325,9 @@ __global__ void __launch_bounds__(256) k_planes(const DevItem* items, int n, int
     const float4* __restrict__ tris = it.tris;
     const int lane = threadIdx.x & 31, n_warps = gridDim.x * (blockDim.x >> 5);
     const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    float reach = 0.0f;                                 // greatest coordinate of the posed mesh
-    for (int k = 0; k < 6; ++k) reach = fmaxf(reach, fabsf(unordered(B.aabb[k])));
+    float far[3];                                       // the farthest corner of the posed mesh's box
+    for (int k = 0; k < 3; ++k) far[k] = fmaxf(fabsf(unordered(B.aabb[k])), fabsf(unordered(B.aabb[3 + k])));
+    const float reach = length(f3(far[0], far[1], far[2]));
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {    // leaves
         const float3 m = unit_or_zero(area_vector(tris, s));
         float h = -INFINITY;

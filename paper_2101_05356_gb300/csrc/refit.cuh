@@ -85,7 +85,9 @@ FR_D float3 unit_or_zero(float3 m) {
 // height h = max n . x over its vertices.  The pad covers the rounding of both
 // sides of the test, a few 2^-24 of the coordinates' magnitude: not of the
 // node's only, since a shadow ray's height is rounded at its origin's, which may
-// lie far beyond the node, so `reach` bounds the whole mesh's.
+// lie far beyond the node, so `reach` bounds the distance of the whole mesh from
+// the camera (17 roundings of it, 1e-6, cover the three products of either dot
+// product, the ends' and the sum's).
 FR_D float4 plane_record(float3 n, float h, float reach) {
     const bool none = n.x == 0.0f && n.y == 0.0f && n.z == 0.0f;
     return make_float4(n.x, n.y, n.z, none ? 1.0f : h + 1e-5f + 1e-6f * reach);
