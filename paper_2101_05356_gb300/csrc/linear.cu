@@ -324,13 +324,12 @@ __global__ void __launch_bounds__(FIN_THREADS) k_linear_adj_finish(const __grid_
 int nb(long n, int t) { return (int)((n + t - 1) / t); }
 
 int sm_count() {
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
+    static const int sms = [] {          // (initialised once, whichever thread's call comes first)
+        int dev = 0, n = 0;
         cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 1;
-    }
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        return std::max(n, 1);
+    }();
     return sms;
 }
 
@@ -406,7 +405,7 @@ void launch_linear_adjoint(const LinearAdjModel* models, int n_models, cudaStrea
         // blocks 0.126, at five, spilling, 0.196 ms; two or four rows' loads in flight
         // at the fewer blocks they leave 0.16-0.18 ms)
         const int most = nb(nb(kmax, 2), LIN_THREADS / 32);
-                const int z = std::max(1, std::min(most, nb(8L * sms, (long)L.start[L.n_models] * n_groups)));
+        const int z = std::max(1, std::min(most, nb(8L * sms, (long)L.start[L.n_models] * n_groups)));
         k_linear_adj_part<LIN_GROUP, 2, 6><<<dim3(L.start[L.n_models], n_groups, z), LIN_THREADS, 0, st>>>(L);
     }
     k_linear_adj_finish<<<dim3(nb(kmax, FIN_K), n, L.n_models), FIN_THREADS, 0, st>>>(L);
