@@ -91,7 +91,7 @@ struct LightDev {
 // Binary BVH node (96 B): both children's boxes and child codes (64 B, four
 // 16-B loads), then each child's plane bound (two more, read by the any-hit
 // traversal): every point x of the child's triangles has n . x <= h, n the
-// child's mean normal (k_planes).
+// child's mean normal (k_pose_refit and k_refit_top; k_planes in the rebuilt tree).
 struct __align__(16) BvhNode {
     float4 a;   // lo0.x lo0.y lo0.z hi0.x
     float4 b;   // hi0.y hi0.z lo1.x lo1.y

@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(256) k_pack(const DevItem* items, int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (n == 1) {
         if (i == 0) {
-            const float4 l = box_leaf[0], h = box_leaf[1];
+            const float4 l = box_leaf[0], h = box_leaf[1];       // one leaf: both children (refit.cu)
             nodes[0].a = make_float4(l.x, l.y, l.z, h.x);
             nodes[0].b = make_float4(h.y, h.z, INFINITY, INFINITY);
             nodes[0].c = make_float4(INFINITY, -INFINITY, -INFINITY, -INFINITY);

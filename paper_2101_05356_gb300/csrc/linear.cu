@@ -227,8 +227,9 @@ __global__ void __launch_bounds__(LIN_THREADS, MIN_BLOCKS) k_linear_adj_part(con
 // it is an L1 hit after the first), which leaves no shared staging to balance
 // over the block's warps.  RB rows' loads are in flight before they are summed,
 // in the same order.  Bound by HBM: 510 MB for both 512 x 512 albedos at K = 80,
-// 75 us; measured 87 us with the second pass, against 119 us with eight columns
-// a warp, one row in flight and five shuffles a sum (four columns: 88 us).
+// 75 us; measured 87 us with the second pass (95 in the benchmark's loop of
+// calls), against 119 us with eight columns a warp, one row in flight and five
+// shuffles a sum (four columns: 88 us).
 constexpr int ONE_K = 2, ONE_ROWS = 4;
 template <int KG, int RB>
 __global__ void __launch_bounds__(LIN_THREADS) k_linear_adj_one(const __grid_constant__ AdjLaunch L) {

@@ -11,7 +11,7 @@
 // memory, every node reduces its own run of them (its leaves are consecutive
 // slots), so there is no order between the nodes and no atomic, and a block
 // poses the vertices it needs itself instead of waiting for another launch.
-// Measured (morph included, paper-scale face): 0.146 -> 0.065 ms; on the 5,120-triangle
+// Measured (morph included, paper-scale face): 0.146 -> 0.067 ms; on the 5,120-triangle
 // face 0.097 -> 0.043 ms.
 #include <algorithm>
 #include <vector>
@@ -236,7 +236,8 @@ FR_D void refit_treelet(const DevItem& it, TreeletShared& sh, const float* R, co
         it.B.treelet_box[3 * k + 1] = make_float4(b.hi.x, b.hi.y, b.hi.z, 0.0f);
         if (tl.up >= 0) {
             store_child(it.nodes[tl.up >> 1], tl.up & 1, b, p);
-        } else if (tl.code < 0) {                 // the tree is one leaf: a root whose second child nothing enters
+        } else if (tl.code < 0) {                 // the tree is one leaf: a root with it as both children
+            // (the second's inverted box is met by every ray, whose slabs it swaps: the leaf is tested twice)
             BvhNode& nd = it.nodes[0];
             nd.a = make_float4(b.lo.x, b.lo.y, b.lo.z, b.hi.x);
             nd.b = make_float4(b.hi.y, b.hi.z, INFINITY, INFINITY);

@@ -350,12 +350,12 @@ FR_D float3 radiance_from(const DevScene& S, const DevParams& P, const SampleSta
     return Lo;
 }
 
-// Warp-cooperative visibility at screen point (sx, sy): the camera ray's hit
-// (without the material) and both shadow-visibility words.
 FR_D void make_cover(const DevScene& S, const SampleState& ss, Cover& c) {
     build_cover(S, c, __ballot_sync(FULL, ss.hit && ss.lit), ss.slot);
 }
 
+// Warp-cooperative visibility at screen point (sx, sy): the camera ray's hit
+// (without the material) and both shadow-visibility words.
 // SPLIT > 1: the block's SPLIT warps hold the same samples; each traces the
 // camera rays and its share of the shadow rays, and all return every bit.
 template <bool ENV, int SPLIT, class C>

@@ -516,7 +516,8 @@ class Renderer:
 
     # Images and losses are stored whole by the library, so the calls below hand
     # it uninitialised buffers: a fill is a launch in front of the call's own
-    # (loss at 512 x 512 33.4 -> 22.2 us a call, 64 x 64 step 244 -> 237 us).
+    # (on one host, loss at 512 x 512 33 -> 22 us a call, most of it host time
+    # that is 22 to 29 us on others; 64 x 64 step 244 -> 237 us).
     def forward(self, dparams, iteration=0, face_id=0):
         img = self.image_output()
         fr_forward(self.ctx, dparams, img, iteration, face_id)
