@@ -58,13 +58,13 @@ OPS_PER_TRI = 30
 # kernel from one ncu capture of this benchmark's workload, valid while the
 # sources that make up the kernel hash to `sources_sha256` (else reported as
 # null); the capture command is recorded beside the kernel's profile summary.
-TRAFFIC = {"k_forward": {"bytes": 20503808 + 793600,
-                         "sources_sha256": "9f4469a1788b8b2e0d8e4da2a3e3d391ba980eb62e4789bc03e618d0c15ea1c1"}}
+TRAFFIC = {"k_forward": {"bytes": 20508416 + 664320,
+                         "sources_sha256": "857da5ce9c7fa5c4eb0128cb5b592d6b300e82b2919bcdd70b4c73bd91d70ee6"}}
 KERNEL_SOURCES = {"k_forward": ("render.cu", "trace.cuh", "shade.cuh", "common.cuh")}
 # Issue-slot use (smsp__issue_active) of a kernel from the same capture,
 # valid while its sources hash to `sources_sha256`.
-ISSUE = {"k_forward": {"frac": 0.7037,
-                       "sources_sha256": "9f4469a1788b8b2e0d8e4da2a3e3d391ba980eb62e4789bc03e618d0c15ea1c1"}}
+ISSUE = {"k_forward": {"frac": 0.7039,
+                       "sources_sha256": "857da5ce9c7fa5c4eb0128cb5b592d6b300e82b2919bcdd70b4c73bd91d70ee6"}}
 FP32_LANES_PER_SM = 128
 
 
