@@ -59,12 +59,12 @@ OPS_PER_TRI = 30
 # sources that make up the kernel hash to `sources_sha256` (else reported as
 # null); the capture command is recorded beside the kernel's profile summary.
 TRAFFIC = {"k_forward": {"bytes": 20508416 + 664320,
-                         "sources_sha256": "857da5ce9c7fa5c4eb0128cb5b592d6b300e82b2919bcdd70b4c73bd91d70ee6"}}
+                         "sources_sha256": "3eca620fc97c503c6e3e999f49b4b8a5cd3123944e639e47022ec9369ed7b0d2"}}
 KERNEL_SOURCES = {"k_forward": ("render.cu", "trace.cuh", "shade.cuh", "common.cuh")}
 # Issue-slot use (smsp__issue_active) of a kernel from the same capture,
 # valid while its sources hash to `sources_sha256`.
 ISSUE = {"k_forward": {"frac": 0.7039,
-                       "sources_sha256": "857da5ce9c7fa5c4eb0128cb5b592d6b300e82b2919bcdd70b4c73bd91d70ee6"}}
+                       "sources_sha256": "3eca620fc97c503c6e3e999f49b4b8a5cd3123944e639e47022ec9369ed7b0d2"}}
 FP32_LANES_PER_SM = 128
 
 

@@ -147,10 +147,12 @@ struct DevParams {
 };
 
 // Fixed-point accumulator layout of G.small: focal, then 3 per light
-// (intensity), then from FR_GEO_OFF 4 per light (d, a, p0, p1), then from
-// FR_ENV_OFF 3 per environment texel.
+// (intensity), then from FR_GEO_OFF 4 per light (d, a, p0, p1), then the part of
+// focal below its resolution (in 2^-64), then from FR_ENV_OFF 3 per environment
+// texel.
 constexpr int FR_GEO_OFF = 1 + 3 * FR_MAX_LIGHTS;
-constexpr int FR_ENV_OFF = FR_GEO_OFF + 4 * FR_MAX_LIGHTS;
+constexpr int FR_FOCAL_LOW = FR_GEO_OFF + 4 * FR_MAX_LIGHTS;
+constexpr int FR_ENV_OFF = FR_FOCAL_LOW + 1;
 constexpr int FR_SMALL = FR_ENV_OFF + 3 * FR_MAX_ENV_D * FR_MAX_ENV_D;
 
 // Gradient sums are kept in 64-bit fixed point (resolution 2^-32, range
@@ -164,6 +166,11 @@ constexpr double FR_FIX_SCALE = 4294967296.0;
 // integer as the FP64 product without using the (narrow) FP64 pipe; measured
 // 6% faster adjoint than the FP64 conversion.  Larger |v| saturates.
 FR_D long long to_fix(float v) { return __float2ll_rn(v * 4294967296.0f); }
+// what to_fix rounds off v, in units of 2^-64
+FR_D long long fix_rest(float v) {
+    const float scaled = v * 4294967296.0f;
+    return fabsf(scaled) < 16777216.0f ? __float2ll_rn((scaled - rintf(scaled)) * 4294967296.0f) : 0ll;
+}
 FR_D long long to_fix_d(double v) { return __double2ll_rn(v * FR_FIX_SCALE); }
 FR_D double from_fix(fix64 v) { return (double)(long long)v * (1.0 / FR_FIX_SCALE); }
 FR_D void fix_add(fix64* a, float v) {

@@ -280,7 +280,8 @@ __global__ void k_pose_finish(const DevItem* items, int NL, int n_blocks) {
             for (int r = 0; r < 3; ++r) s += R[3 * c2 + r] * acc12[9 + r];
             if (it.g_trans) it.g_trans[c2] += (float)(-s);
         }
-        if (it.g_focal) it.g_focal[0] += (float)from_fix(small[0]);
+        if (it.g_focal)
+            it.g_focal[0] += (float)(from_fix(small[0]) + from_fix(small[FR_FOCAL_LOW]) * (1.0 / FR_FIX_SCALE));
     }
     if (it.g_light)
         for (int k = t; k < 3 * NL; k += blockDim.x) it.g_light[k] += (float)from_fix(small[1 + k]);

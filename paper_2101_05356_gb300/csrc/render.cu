@@ -1182,15 +1182,20 @@ __global__ void __launch_bounds__(RT_THREADS, FR_EDGE_MIN_BLOCKS) k_edge_primary
     }
     scatter_vertex(G.d_v, E.x, gA, active);
     scatter_vertex(G.d_v, E.y, gB, active);
-    // each warp's sum is rounded to fixed point by itself, so the total is the same
-    // whether a block holds four warps of samples or (SPLIT) one
+    // each warp's sum enters the total by itself, in two words that hold it exactly,
+    // so the total is the same whether a block holds four warps of samples or (SPLIT)
+    // one, and rounded once
     const float gw = warp_sum(gf);
     if ((threadIdx.x & 31) == 0) acc_dyn[threadIdx.x >> 5] = gw;
     __syncthreads();
     if (threadIdx.x == 0) {
-        long long s = 0;
-        for (int w = 0; w < RT_WARPS; ++w) s += to_fix_d((double)acc_dyn[w]);
+        long long s = 0, rest = 0;
+        for (int w = 0; w < RT_WARPS; ++w) {
+            s += to_fix(acc_dyn[w]);
+            rest += fix_rest(acc_dyn[w]);
+        }
         if (s != 0) atomicAdd(&G.small[0], (fix64)s);
+        if (rest != 0) atomicAdd(&G.small[FR_FOCAL_LOW], (fix64)rest);
     }
 }
 

@@ -42,6 +42,25 @@ def test_focal_gradient_alone_and_in_a_batch(n_lights):
     assert r.status() == 0
 
 
+@pytest.mark.parametrize("width,height", [(48, 40), (331, 290)])
+def test_focal_gradient_is_linear_in_the_lights(width, height):
+    """The primary edges' focal gradient under lights dimmed by 2^-20 is 2^-20 of the gradient (every product scales
+    exactly): sums kept to 2^-32 would be off by 1e-4 of it, kept to 2^-64 the FP32 result's rounding is left."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2101_05356_gb300 import facert
+    sc = synth.make_scene("tiny", width=width, height=height, n_lights=40)
+    r = facert.Renderer(sc, flags=facert.FLAG_NO_INTERIOR | facert.FLAG_NO_SHADOW_EDGE | facert.FLAG_NO_SPECULAR_EDGE)
+    pr = synth.random_params(sc, 1)
+    adj = torch.randn(height, width, 3, generator=torch.Generator().manual_seed(0)).cuda()
+    g = []
+    for scale in (1.0, 2.0 ** -20):
+        p = r.device_params(pr)
+        p["light_i"] = p["light_i"] * scale
+        g.append(float(r.backward(p, adj, iteration=1)["focal"]) / scale)
+    assert abs(g[0]) > 0.0 and abs(g[1] - g[0]) <= 2e-7 * abs(g[0]), g
+
+
 @pytest.mark.parametrize("spp", [1, 2, 4, 32])
 @pytest.mark.parametrize("n_lights", [2, 5, 11, 40, 66])
 def test_image_alone_and_in_a_batch(n_lights, spp):
